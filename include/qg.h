@@ -284,10 +284,11 @@ qg_status qg_set_solver(qg_handle h, qg_solver kind, int32_t cycles);
  * the tensor cores, 3xTF32 (FP32 grids of at most 64 x 128 or 128 x 64
  * intervals with one layer, 64 x 64 with two: both layers' transforms and
  * the coupled solve of Eqs. isub-1/2 per mode); 41: the same products with tcgen05.mma and TMEM
- * accumulators (sides of 16 to 64 intervals); 50: radix-16 FFT passes with the values in
- * registers, one to four sequence pairs per CTA and three launches (one
- * per pass), for elliptic grids of 256 to 8192 intervals a side (4096 in
- * FP64); 0:
+ * accumulators (sides of 16 to 64 intervals); 50: half-length sine
+ * transforms (radix-16 passes with the values in registers, only the half
+ * that the odd symmetry leaves), several sequence pairs per CTA and three
+ * launches (one per pass), for elliptic grids of 128 to 8192 intervals a side (4096 in
+ * FP64) above 128 x 128; 0:
  * the multigrid solver (qg_set_solver).  These are
  * implementations of the same sine-transform solve of Section 4.3, equal to
  * rounding.  No device work.  Errors: QG_ERR_ARG.                          */

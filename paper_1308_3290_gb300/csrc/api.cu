@@ -51,6 +51,9 @@ struct LevelTables {
     void* lamy = nullptr;  // (2 cos(pi l/my) - 2)/dyc^2, l = 0..my
     void* ptx[3] = {nullptr, nullptr, nullptr};  // warp-group engine pass twiddles for
     void* pty[3] = {nullptr, nullptr, nullptr};  //   L = 2 mx and 2 my, engines 32/33/34
+    void* htx = nullptr;                         // engine 50: twiddles for L = 2 mx and
+    void* hty = nullptr;                         //   2 my, and the y eigenvalues in the
+    void* lamyr = nullptr;                       //   order of its rows
     void* mtab = nullptr;  // matrix engine (FP32, one layer): sine matrices and 1/lambda
     void* tctab = nullptr; // engine 41: split sine matrices (shared-memory image), 1/lambda
 };
@@ -314,6 +317,29 @@ qg_status get_pass_table(qg_ctx* h, int L, int rad, void** out) {
     return QG_OK;
 }
 
+// The twiddle table of engine 50 for length L (half_table).
+qg_status get_half_table(qg_ctx* h, int L, void** out) {
+    const int key = -(L * 64 + 63);   // shares the twiddle cache with the pass tables
+    auto it = h->twcache.find(key);
+    if (it != h->twcache.end()) {
+        *out = it->second;
+        return QG_OK;
+    }
+    const size_t n = half_table_size(L);
+    std::vector<double> re(n), im(n), v(2 * n);
+    half_table(L, re.data(), im.data());
+    for (size_t k = 0; k < n; ++k) {
+        v[2 * k] = re[k];
+        v[2 * k + 1] = im[k];
+    }
+    void* d = nullptr;
+    qg_status s = upload_real(h, &d, v);
+    if (s != QG_OK) return s;
+    h->twcache[key] = d;
+    *out = d;
+    return QG_OK;
+}
+
 // Eigenvalue and twiddle tables of grid level `lv` (Eq. ialpha without Ro).
 qg_status get_level(qg_ctx* h, int lv, const LevelTables** out) {
     auto it = h->tables.find(lv);
@@ -334,10 +360,7 @@ qg_status get_level(qg_ctx* h, int lv, const LevelTables** out) {
     if (s == QG_OK) s = get_twiddles(h, t.my, &t.twy);
     for (int r = 0; r < 3 && s == QG_OK; ++r) {
         const int rad = warp_engine_radix(32 + r);
-        // radix 16 (r = 1) also serves engine 50
-        if (!solve32_supports(t.mx, t.my, rad, h->esz) &&
-            !(rad == 16 && stream_supports(t.mx, t.my, h->esz)))
-            continue;
+        if (!solve32_supports(t.mx, t.my, rad, h->esz)) continue;
         s = get_pass_table(h, 2 * t.mx, rad, &t.ptx[r]);
         if (s == QG_OK) s = get_pass_table(h, 2 * t.my, rad, &t.pty[r]);
     }
@@ -365,6 +388,13 @@ qg_status get_level(qg_ctx* h, int lv, const LevelTables** out) {
     for (int l = 1; l < t.my; ++l) ly[l] = (2.0 * std::cos(pi * l / t.my) - 2.0) / (t.dyc * t.dyc);
     s = upload_real(h, &t.lamx, lx);
     if (s == QG_OK) s = upload_real(h, &t.lamy, ly);
+    if (s == QG_OK && stream_supports(t.mx, t.my, h->esz)) {
+        s = get_half_table(h, 2 * t.mx, &t.htx);
+        if (s == QG_OK) s = get_half_table(h, 2 * t.my, &t.hty);
+        std::vector<double> lr((size_t)9 * (t.my / 8));
+        half_lam(t.my, ly.data(), lr.data());
+        if (s == QG_OK) s = upload_real(h, &t.lamyr, lr);
+    }
     if (s != QG_OK) return s;
     h->tables[lv] = t;
     *out = &h->tables[lv];
@@ -529,10 +559,13 @@ qg_status solve_level(qg_ctx* h, const LevelTables& t, const void* in, void* tr,
     P.twx = static_cast<const C*>(t.twx);
     P.twy = static_cast<const C*>(t.twy);
     const int eng = engine ? engine : engine_for(h, t.mx, t.my);
-    const int tab = eng == kStreamEngine ? 1 : eng - 32;   // engine 50: radix-16 tables
-    const bool fft_tab = is_warp_engine(eng) || eng == kStreamEngine;
-    P.ptx = fft_tab ? static_cast<const C*>(t.ptx[tab]) : nullptr;
-    P.pty = fft_tab ? static_cast<const C*>(t.pty[tab]) : nullptr;
+    if (is_warp_engine(eng)) {
+        P.ptx = static_cast<const C*>(t.ptx[eng - 32]);
+        P.pty = static_cast<const C*>(t.pty[eng - 32]);
+    }
+    P.htx = static_cast<const C*>(t.htx);
+    P.hty = static_cast<const C*>(t.hty);
+    P.lamyr = static_cast<const T*>(t.lamyr);
     P.lamx = static_cast<const T*>(t.lamx);
     P.lamy = static_cast<const T*>(t.lamy);
     P.scale = (T)((2.0 / t.mx) * (2.0 / t.my));
@@ -570,7 +603,7 @@ qg_status solve_level(qg_ctx* h, const LevelTables& t, const void* in, void* tr,
 // values per thread, engines 32, 33, 34; or, on small one-layer FP32 grids,
 // the matrix-form solve on the tensor cores of solve_mtx.cu, engine 40, or
 // the same with tcgen05 and TMEM accumulators, engine 41 (solve_tc.cu); or
-// the register-resident radix-16 passes of solve_stream.cu, engine 50) is
+// the half-length sine transforms of solve_stream.cu, engine 50) is
 // chosen per handle when it is created, by timing a few whole steps with each
 // engine that supports the elliptic grid (the solve alone, timed back to
 // back, ranks them differently: in a step the fine sweep has just streamed
@@ -594,7 +627,7 @@ int engine_for(qg_ctx* h, int mx, int my) {
 bool engine_ok(const qg_ctx* h, const LevelTables* t, size_t esz, int e) {
     if (e == kMatrixEngine) return t->mtab && mtx_supports(t->mx, t->my, esz, h->layers);
     if (e == kTcEngine) return t->tctab && tc_supports(t->mx, t->my, esz, h->layers);
-    if (e == kStreamEngine) return solve_engine_supports(t->mx, t->my, esz, e) && t->ptx[1];
+    if (e == kStreamEngine) return solve_engine_supports(t->mx, t->my, esz, e) && t->htx;
     return solve_engine_supports(t->mx, t->my, esz, e) && (!is_warp_engine(e) || t->ptx[e - 32]);
 }
 
@@ -1469,14 +1502,17 @@ qg_status qg_poisson_solve(qg_handle h, const void* rhs, void* psi, int level) {
     const size_t pl = (size_t)(t->my + 1) * t->ldc;
     const int ld_tr = padded_ld(t->my);
     const size_t pl_tr = (size_t)(t->mx + 1) * ld_tr;
-    // (the multigrid path keeps its result in the second part)
-    const size_t bytes = (pl + (pl_tr > pl ? pl_tr : pl)) * h->layers * h->esz;
+    // (the multigrid path keeps its result in the second part; two layers
+    // keep their output apart from the scratch, see kStreamEngine)
+    const size_t part2 = (pl_tr > pl ? pl_tr : pl) * h->layers * h->esz;
+    const size_t apart = h->layers == 2 ? pl * h->layers * h->esz : 0;
+    const size_t bytes = pl * h->layers * h->esz + part2 + apart;
     void* buf = nullptr;
     QG_TRY(cudaMallocAsync(&buf, bytes, h->stream));
     void* tbuf = static_cast<char*>(buf) + pl * h->layers * h->esz;
     cudaError_t e = cudaMemsetAsync(buf, 0, bytes, h->stream);
     const size_t dense = (size_t)(t->mx - 1) * (t->my - 1) * h->esz;
-    void* buf_out = buf;
+    void* buf_out = apart ? static_cast<char*>(tbuf) + part2 : buf;
     for (int L = 0; L < h->layers && e == cudaSuccess; ++L)
         e = copy_in(static_cast<char*>(buf) + L * pl * h->esz, t->ldc,
                     static_cast<const char*>(rhs) + L * dense, t->mx - 1, t->my - 1,
@@ -1489,8 +1525,8 @@ qg_status qg_poisson_solve(qg_handle h, const void* rhs, void* psi, int level) {
         buf_out = tbuf;
     } else if (e == cudaSuccess) {
         s = h->dtype == QG_F64
-                ? solve_level<double>(h, *t, buf, tbuf, ld_tr, pl_tr, buf, buf, pl, h->stream)
-                : solve_level<float>(h, *t, buf, tbuf, ld_tr, pl_tr, buf, buf, pl, h->stream);
+                ? solve_level<double>(h, *t, buf, tbuf, ld_tr, pl_tr, buf, buf_out, pl, h->stream)
+                : solve_level<float>(h, *t, buf, tbuf, ld_tr, pl_tr, buf, buf_out, pl, h->stream);
         if (s != QG_OK) e = cudaErrorUnknown;
     }
     for (int L = 0; L < h->layers && e == cudaSuccess; ++L)
@@ -2434,11 +2470,13 @@ qg_status group_solve(qg_ensemble e, const EnsSolveGroup& g, int engine, int k, 
     P.ld_tr = h0->ld_t;
     P.twx = static_cast<const C*>(t->twx);
     P.twy = static_cast<const C*>(t->twy);
-    if (is_warp_engine(engine) || engine == kStreamEngine) {
-        const int tab = engine == kStreamEngine ? 1 : engine - 32;   // engine 50: radix 16
-        P.ptx = static_cast<const C*>(t->ptx[tab]);
-        P.pty = static_cast<const C*>(t->pty[tab]);
+    if (is_warp_engine(engine)) {
+        P.ptx = static_cast<const C*>(t->ptx[engine - 32]);
+        P.pty = static_cast<const C*>(t->pty[engine - 32]);
     }
+    P.htx = static_cast<const C*>(t->htx);
+    P.hty = static_cast<const C*>(t->hty);
+    P.lamyr = static_cast<const T*>(t->lamyr);
     P.lamx = static_cast<const T*>(t->lamx);
     P.lamy = static_cast<const T*>(t->lamy);
     P.scale = (T)((2.0 / t->mx) * (2.0 / t->my));

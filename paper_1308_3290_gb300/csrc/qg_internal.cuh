@@ -72,6 +72,9 @@ struct SolveParams {
     const typename Cx<T>::type* twy;   // e^{i pi t/my}, t < 2 my
     const typename Cx<T>::type* ptx;   // warp-group engine: per-pass twiddles for
     const typename Cx<T>::type* pty;   //   2 mx and 2 my (see pass_table_size)
+    const typename Cx<T>::type* htx;   // engine 50: half_table(2 mx) and
+    const typename Cx<T>::type* hty;   //   half_table(2 my)
+    const T* lamyr;                     // engine 50: lamy in its rows' order (half_lam)
     const T* lamx;                      // (2 cos(pi k/mx) - 2)/dx^2, k = 0..mx
     const T* lamy;                      // (2 cos(pi l/my) - 2)/dy^2, l = 0..my
     T scale, Ro, f1, f2;
@@ -114,10 +117,15 @@ bool solve32_supports(int mx, int my, int rad, size_t esz);
 // engines 32, 33, 34: the warp-group engine with 32, 16, 8 values per thread
 inline int warp_engine_radix(int engine) { return engine == 34 ? 8 : (engine == 33 ? 16 : 32); }
 inline bool is_warp_engine(int engine) { return engine >= 32 && engine <= 34; }
-// engine 50: one CTA per sequence pair, three launches, radix-16 passes
-// with the values in registers (solve_stream.cu); it takes the radix-16
-// pass tables of engine 33 (ptx/pty)
+// engine 50: half-length sine transforms, radix-16 passes with the values in
+// registers, three launches (solve_stream.cu); tr and work are scratch in its
+// own layouts, and with two layers out may not alias work
 constexpr int kStreamEngine = 50;
+// its twiddle table for L = 2N, and the eigenvalues lam[0..M] of a direction
+// of M intervals in the order of its rows (9 M/8 values)
+size_t half_table_size(int L);
+void half_table(int L, double* re, double* im);
+void half_lam(int M, const double* lam, double* out);
 bool stream_supports(int mx, int my, size_t esz);
 template <typename T>
 cudaError_t launch_solve_stream(const SolveParams<T>& P, cudaStream_t s);

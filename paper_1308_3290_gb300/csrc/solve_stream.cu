@@ -1,45 +1,57 @@
-// Elliptic solve of Section 4.3 for long sequences (engine 50).
+// Elliptic solve of Section 4.3 with half-length sine transforms (engine 50).
 //
-// The same transforms as the warp-group engine of solve32.cu: the x pass of
-// the right-hand side, the y pass with the mode-space solve of Eq. ialpha
-// (or Eqs. isub-1/2 for two layers), and the inverse x pass, each a DST-I
-// of two real sequences computed as one complex FFT of length L = 2N of
-// their odd extensions (F(a)_k = -Im Z_k / 2, F(b)_k = Re Z_k / 2).  The
-// engine is laid out for grids whose passes stream through HBM (the full
-// 2048 x 4096 grid, l = 0):
+// The x pass of the right-hand side, the y pass with the mode-space solve of
+// Eq. ialpha (or Eqs. isub-1/2 for two layers), and the inverse x pass.  Each
+// is a DST-I of two real sequences a, b at once, z = a + i b, defined through
+// the FFT of length L = 2N of the odd extension of z (Z_k = -2i F_k, so
+// F(a)_k = -Im Z_k / 2, F(b)_k = Re Z_k / 2), but only the half that the odd
+// symmetry leaves is computed:
 //
-//   * G = L/16 threads per sequence pair, three plain launches (one per
-//     pass) chained by programmatic dependent launch, so there is no grid
-//     barrier and each pass takes the CTA size and register budget of its
-//     own length; an ensemble group's batch runs instead as one launch, a
-//     work queue over the items of the three passes of every member
-//     (stream_queue_kernel);
-//   * thread t holds the 16 values x[t + G r] in registers.  The first
-//     radix-16 pass works on the values the thread loaded from global
-//     memory, and the last pass leaves X[t + G s] in registers (a Stockham
-//     pass of sub-transform size L/16 writes its output in natural order),
-//     so an FFT of length L = 16^p 2^q takes p + (q > 0) - 1 shared-memory
-//     exchanges (L = 4096: two; 8192: three) between the global load and
-//     the global store;
-//   * the odd extension is completed in shared memory: each thread stores
-//     its z[t + G r], r < 8, and reads back the reflected -z[L - m];
-//   * the y pass keeps the forward spectrum in registers for the mode-space
-//     solve and starts the inverse transform from there;
-//   * one shared buffer of L complex per pair: every pass reads all its
-//     operands into registers before any thread of the pair writes;
-//   * the passes that write transposed (x forward into tr, y into work) hold
-//     2 or 4 pairs per CTA, each on its own named barrier, and stage their
-//     outputs in shared memory so that each row receives 2 PPC consecutive
-//     values (FP32, 4 pairs: a whole 32-byte sector) instead of one 8-byte
-//     pair per row and thread;
-//   * the length is a template parameter: every shared-memory, twiddle and
-//     global offset of a pass is a constant from a per-thread base.
+//   * with G = L/16, butterfly t of the first radix-16 pass takes x[t + G r],
+//     r < 16, which are z[t + G r], r < 8, and -z[c G - t], c = 16 - r <= 8:
+//     no odd extension is ever stored.  Butterfly G - t is that of t with its
+//     inputs reversed and negated, Y_{G-t}[s] = -e^{2 pi i s/16} Y_t[-s], so
+//     only t = 0 .. G/2 are computed;
+//   * the sixteen sub-transforms of length G that follow, over
+//     u_s[t] = e^{-2 pi i t s/L} Y_t[s], give X[s + 16 k]; by u_s[G - t] =
+//     -u_{-s}[t] and X[L - m] = -X[m] the rows s = 1..7 also hold the rows
+//     16 - s, so only rows s = 0..8 are computed (rows 0 and 8 are their own
+//     images and come out twice: 9/16 of the work instead of 1/2).
 //
-// Twiddles come from the radix-16 pass tables of the warp-group engine
-// (pass_table(L, 16), FP64-generated): a radix-16 pass loads w, w^2, w^4
-// and w^8 and forms the other powers, the remainder pass one power per
-// radix and multiplies by 16th roots of unity.
+// The sine sum is symmetric, so the same factors in the opposite order
+// (rows first, then the radix-16 pass over s) transform from the rows' order
+// back to natural order.  Every output is a sum of products with unit-modulus
+// factors (no running sum, no division by a sine), so the rounding error
+// grows like log N as for the full-length FFT.
+//
+// Layout of the work: a pair of sequences has 9 G/16 threads.  In the radix-16
+// pass thread t <= G/2 does butterfly t; in the rows thread (s, j), j < H =
+// G/16, holds 16 values u_s[j + H r], does a 16-point DFT, exchanges with the
+// H threads of its row (a warp or less, so no CTA barrier below L = 16384)
+// and finishes with H-point DFTs (H = 32, 64: 8 x 4, 16 x 4, one more
+// exchange).  One CTA barrier lies between the pass and the rows.
+//
+//   x forward: pass, rows;        modes in position order -> tr
+//   y:         pass, rows, mode-space solve, rows, pass  -> work
+//   x inverse: rows, pass                                -> out
+//
+// An x-mode m = s + 16 k (k < G/2) has position s G/2 + k: the order in
+// which the inverse x pass's rows read, so that its loads are contiguous.
+// tr and work are scratch arrays and interleave the two sequences of the
+// pass that reads them (tr: [pair of positions][row][2]; work: [pair of
+// rows][position][2]; two layers: [position][row][layer] and
+// [row][position][layer]), so a pass loads z as one vector and the pass
+// before writes runs of 4 values a pair: 32-byte sectors from two pairs on.
+//
+// Three launches chained by programmatic dependent launch; an ensemble group's
+// batch runs as one launch, a work queue over the items of the three passes
+// of every member (stream_queue_kernel).
+//
+// All twiddles come from one FP64-generated table per length (half_table):
+// every factor is a rounded exact value.
 #include <cuda_runtime.h>
+
+#include <cmath>
 
 #include "bounds.cuh"
 #include "dst_engine.cuh"
@@ -50,21 +62,33 @@ namespace {
 
 using namespace eng;
 
-// padded slot of complex element m (one pad per 16 spreads the strided
-// stores of the passes over the banks)
-__host__ __device__ constexpr int sp(int m) { return m + (m >> 4); }
-__host__ __device__ constexpr int buf_elems(int L) { return sp(L) + 2; }
+// Geometry of a length L = 2^LG = 2N.
+template <int LG>
+struct Half {
+    static constexpr int L = 1 << LG, N = L / 2, G = L / 16, H = G / 16;
+    static constexpr int HC = H <= 16 ? 1 : 4, HB = H / HC;   // the rows' second DFTs
+    static constexpr int TP = 9 * H;                          // threads per pair
+    static constexpr int P2 = H + 1;   // pitch of a row's exchange [q][j], q < 16, j < H
+    // pitch of a row: 16 P2 = G + 16, and more where several rows share a
+    // half warp, so that their lanes fall on different banks
+    static constexpr int RP = H == 1 ? 17 : 16 * P2 + (H <= 8 ? H : 0);
+    static constexpr int BUF = 9 * RP;                        // complex elements per pair
+    // table: T1[s - 1][t] = e^{-2 pi i t s/L}, s = 1..8, t <= G/2 (pitch PT);
+    // T2[q - 1][j] = e^{-2 pi i q j/G}, q = 1..15, j < H;
+    // T3[p][c] = e^{-2 pi i p c/H}, p < HB, c < HC (HC > 1)
+    static constexpr int PT = G / 2 + 2;
+    static constexpr int T2 = 8 * PT, T3 = T2 + 15 * H, TABLE = T3 + (HC > 1 ? H : 0);
+};
 
-// Shared-memory access at padded slot i (a slot, not an element index).
 template <typename T>
-__device__ __forceinline__ Cplx<T> ldsl(const CT<T>* b, int i, int lim) {
+__device__ __forceinline__ Cplx<T> lds_(const CT<T>* b, int i, int lim) {
     (void)lim;
     if (!QG_IN(i, lim, 61)) return Cplx<T>{T(0), T(0)};
     const CT<T> v = b[i];
     return Cplx<T>{v.x, v.y};
 }
 template <typename T>
-__device__ __forceinline__ void stsl(CT<T>* b, int i, Cplx<T> v, int lim) {
+__device__ __forceinline__ void sts_(CT<T>* b, int i, Cplx<T> v, int lim) {
     (void)lim;
     if (!QG_IN(i, lim, 62)) return;
     CT<T> w;
@@ -72,439 +96,554 @@ __device__ __forceinline__ void stsl(CT<T>* b, int i, Cplx<T> v, int lim) {
     w.y = v.y;
     b[i] = w;
 }
-
-// FFT length L = 2^LG = 16^NP 2^REM, G = L/16 threads per pair (LG >= 8, so
-// G is a multiple of 16 and sp(a + r G) = sp(a) + r sp(G) for a < G).
-template <int LG>
-struct Len {
-    static constexpr int L = 1 << LG, N = L / 2, G = L / 16, NP = LG / 4, REM = LG % 4;
-    static constexpr int LIM = buf_elems(L);
-    static constexpr int SG = G + G / 16;   // sp(G)
-};
-
-// Barrier of the G threads of one pair (named barrier 1 + group), or of the
-// whole CTA when it holds one pair.
-struct GSync {
-    int id, n;
-    bool cta;
-    __device__ __forceinline__ void sync() const {
-        if (cta) __syncthreads();
-        else asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
-    }
-};
-
-// Offset of pass p's block in pass_table(L, 16): blocks of 16 x 16^q for
-// q = 1 .. p - 1.
-__host__ __device__ constexpr int tw_off(int p) {
-    int o = 0, ns = 16;
-    for (int q = 1; q < p; ++q, ns *= 16) o += 16 * ns;
-    return o;
-}
-
-// Store the outputs of radix-16 pass q (sub-transform size NS = 16^q) to
-// (t - k) 16 + k + r NS, k = t mod NS, in padded slots.
-template <typename T, int LG, int NS>
-__device__ __forceinline__ void put_pass(const Cplx<T> (&v)[16], CT<T>* buf, int t) {
-    using Ln = Len<LG>;
-    int base;
-    if constexpr (NS == 1) {
-        base = 17 * t;                      // sp(16 t + r) = 17 t + r
-    } else {
-        const int k = t & (NS - 1);
-        const int d = (t - k) * 16 + k;
-        base = d + (d >> 4);                // sp(d + r NS) = sp(d) + r sp(NS)
-    }
-    constexpr int step = NS == 1 ? 1 : NS + NS / 16;
-#pragma unroll
-    for (int r = 0; r < 16; ++r) stsl<T>(buf, base + r * step, v[out_slot<16>(r)], Ln::LIM);
-}
-
-// Radix-16 pass p >= 1 (sub-transform size 16^p): read t + r G, twiddle,
-// 16-point DFT.
-template <typename T, int LG, int P>
-__device__ __forceinline__ void mid_pass(Cplx<T> (&v)[16], CT<T>* buf, int t,
-                                         const CT<T>* __restrict__ tw, const GSync& sy) {
-    using Ln = Len<LG>;
-    constexpr int NS = 1 << (4 * P);
-    put_pass<T, LG, NS / 16>(v, buf, t);
-    sy.sync();
-    const int rb = t + (t >> 4);
-#pragma unroll
-    for (int r = 0; r < 16; ++r) v[r] = ldsl<T>(buf, rb + r * Ln::SG, Ln::LIM);
-    sy.sync();
-    // twiddles w^r = e^{-2 pi i r k / (16 NS)}: w, w^2, w^4 and w^8 from the
-    // table, the other powers as products (at most three roundings deep)
-    const CT<T>* tp = tw + tw_off(P) + (t & (NS - 1));
-    Cplx<T> w[16];
-    {
-        const CT<T> a = __ldg(tp + NS), b = __ldg(tp + 2 * NS), c = __ldg(tp + 4 * NS),
-                    d = __ldg(tp + 8 * NS);
-        w[1] = Cplx<T>{a.x, a.y};
-        w[2] = Cplx<T>{b.x, b.y};
-        w[4] = Cplx<T>{c.x, c.y};
-        w[8] = Cplx<T>{d.x, d.y};
-    }
-    w[3] = cmul(w[2], w[1].x, w[1].y);
-    w[5] = cmul(w[4], w[1].x, w[1].y);
-    w[6] = cmul(w[4], w[2].x, w[2].y);
-    w[7] = cmul(w[4], w[3].x, w[3].y);
-#pragma unroll
-    for (int r = 1; r < 8; ++r) w[8 + r] = cmul(w[8], w[r].x, w[r].y);
-#pragma unroll
-    for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], w[r].x, w[r].y);
-    dft<T, 16>(v);
-}
-
-// e^{-2 pi i m / 16}, m = 0..15, as compile-time constants
+// a conj(w)
 template <typename T>
-__device__ __forceinline__ Cplx<T> w16(int m) {
-    const T c1 = K16<T>::c1, s1 = K16<T>::s1, r2 = K16<T>::r2;
-    const T cs[4] = {T(1), c1, r2, s1}, sn[4] = {T(0), s1, r2, c1};
-    const int q = m >> 2, e = m & 3;
-    const T c = cs[e], s = sn[e];   // e^{-i pi e / 8} = c - i s
-    switch (q) {                    // times (-i)^q
-        case 0: return Cplx<T>{c, -s};
-        case 1: return Cplx<T>{-s, -c};
-        case 2: return Cplx<T>{-c, s};
-        default: return Cplx<T>{s, c};
+__device__ __forceinline__ Cplx<T> cmulc(Cplx<T> a, Cplx<T> w) {
+    return {a.x * w.x + a.y * w.y, a.y * w.x - a.x * w.y};
+}
+template <typename T>
+__device__ __forceinline__ Cplx<T> ldt(const CT<T>* t, int i, int lim) {
+    (void)lim;
+    if (!QG_IN(i, lim, 68)) return Cplx<T>{T(1), T(0)};
+    const CT<T> v = __ldg(t + i);
+    return Cplx<T>{v.x, v.y};
+}
+
+// The outputs of dft<R> in natural order.
+template <typename T, int R>
+__device__ __forceinline__ void dft_nat(Cplx<T>* v) {
+    dft<T, R>(v);
+    if constexpr (R >= 8) {
+        Cplx<T> o[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) o[r] = v[out_slot<R>(r)];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = o[r];
     }
 }
 
-// The remainder pass (radix R = 2^REM, B = 16/R butterflies j = t + b G per
-// thread, sub-transform size L/R): output X[t + G (b + B r)] to v[b + B r].
-template <typename T, int LG, int R>
-__device__ __forceinline__ void rem_pass(Cplx<T> (&v)[16], CT<T>* buf, int t,
-                                         const CT<T>* __restrict__ tw, const GSync& sy) {
-    using Ln = Len<LG>;
-    constexpr int B = 16 / R, NSR = Ln::L / R, SNSR = NSR + NSR / 16;
-    put_pass<T, LG, (1 << (4 * Ln::NP)) / 16>(v, buf, t);
-    sy.sync();
-    const int rb = t + (t >> 4);
-    Cplx<T> u[B][R];
+// Threads of one row: a warp's lanes (H <= 32), else (H = 64) two warps,
+// which meet at the CTA barrier (every thread of the CTA runs the same
+// stages).
+template <int LG>
+__device__ __forceinline__ void row_sync() {
+    if constexpr (Half<LG>::H > 32) __syncthreads();
+    else if constexpr (Half<LG>::H > 1) __syncwarp();
+}
+
+// Radix-16 pass: v[r] = x[t + G r] -> u_s[t] and u_s[G - t] of the rows
+// s = 0..8 in buf (t <= G/2).
+template <typename T, int LG>
+__device__ __forceinline__ void pass_fwd(Cplx<T> (&v)[16], CT<T>* buf, int t,
+                                         const CT<T>* __restrict__ tab) {
+    using Q = Half<LG>;
+    dft_nat<T, 16>(v);
+    const bool both = t > 0 && t < Q::G / 2;
 #pragma unroll
-    for (int b = 0; b < B; ++b)
-#pragma unroll
-        for (int r = 0; r < R; ++r) u[b][r] = ldsl<T>(buf, rb + b * Ln::SG + r * SNSR, Ln::LIM);
-    sy.sync();
-    // twiddle of butterfly j = t + b G: e^{-2 pi i r j / L} = e^{-2 pi i r t / L}
-    // e^{-2 pi i r b / 16} (G = L / 16): R - 1 table loads per thread
-    const CT<T>* tp = tw + tw_off(Ln::NP) + t;
-    Cplx<T> wt[R];
-#pragma unroll
-    for (int r = 1; r < R; ++r) {
-        const CT<T> a = __ldg(tp + r * NSR);
-        wt[r] = Cplx<T>{a.x, a.y};
-    }
-#pragma unroll
-    for (int b = 0; b < B; ++b) {
-#pragma unroll
-        for (int r = 1; r < R; ++r) {
-            const Cplx<T> c = w16<T>((r * b) & 15);
-            const Cplx<T> w = b == 0 ? wt[r] : cmul(wt[r], c.x, c.y);
-            u[b][r] = cmul(u[b][r], w.x, w.y);
+    for (int s = 0; s <= 8; ++s) {
+        Cplx<T> a = v[s], b = v[(16 - s) & 15];
+        if (s > 0) {
+            const Cplx<T> w = ldt<T>(tab, (s - 1) * Q::PT + t, Q::TABLE);
+            a = cmul(a, w.x, w.y);
+            b = cmulc(b, w);
         }
-        dft<T, R>(u[b]);
-#pragma unroll
-        for (int r = 0; r < R; ++r) v[b + B * r] = u[b][out_slot<R>(r)];
+        sts_<T>(buf, s * Q::RP + t, a, Q::BUF);
+        if (both) sts_<T>(buf, s * Q::RP + Q::G - t, Cplx<T>{-b.x, -b.y}, Q::BUF);
     }
 }
 
-// Forward FFT of length L: on entry v[r] = x[t + G r], on return
-// v[s] = X[t + G s].  buf is free on entry and on return.
+// The transposed pass: rows V_s[t], V_s[G - t] in buf -> v[r] = z[t + G r]
+// (r >= 8: -z[(16 - r) G - t]), t <= G/2.
 template <typename T, int LG>
-__device__ __forceinline__ void fft16s(Cplx<T> (&v)[16], CT<T>* buf, int t,
-                                       const CT<T>* __restrict__ tw, const GSync& sy) {
-    using Ln = Len<LG>;
-    dft<T, 16>(v);   // pass 0: sub-transform size 1, no twiddles
-    if constexpr (Ln::NP >= 2) mid_pass<T, LG, 1>(v, buf, t, tw, sy);
-    if constexpr (Ln::NP >= 3) mid_pass<T, LG, 2>(v, buf, t, tw, sy);
-    if constexpr (Ln::REM == 0) {
-        // the last radix-16 pass had sub-transform size G: X[t + G r] is in
-        // slot out_slot(r)
-        Cplx<T> o[16];
+__device__ __forceinline__ void pass_bwd(Cplx<T> (&v)[16], const CT<T>* buf, int t,
+                                         const CT<T>* __restrict__ tab) {
+    using Q = Half<LG>;
+    const int tm = t == 0 ? 0 : Q::G - t;
+    v[0] = lds_<T>(buf, t, Q::BUF);
 #pragma unroll
-        for (int r = 0; r < 16; ++r) o[r] = v[out_slot<16>(r)];
-#pragma unroll
-        for (int r = 0; r < 16; ++r) v[r] = o[r];
+    for (int s = 1; s <= 8; ++s) {
+        const Cplx<T> w = ldt<T>(tab, (s - 1) * Q::PT + t, Q::TABLE);
+        const Cplx<T> a = lds_<T>(buf, s * Q::RP + t, Q::BUF);
+        v[s] = cmul(a, w.x, w.y);
+        if (s < 8) {
+            const Cplx<T> b = cmulc(lds_<T>(buf, s * Q::RP + tm, Q::BUF), w);
+            v[16 - s] = Cplx<T>{-b.x, -b.y};
+        }
+    }
+    dft_nat<T, 16>(v);
+}
+
+// The index k (of X[s + 16 k]) of register i of thread j of a row.
+template <int LG>
+__device__ __forceinline__ int row_k(int j, int i) {
+    using Q = Half<LG>;
+    if constexpr (Q::HC == 1) {
+        return j + (i / Q::H) * Q::H + 16 * (i % Q::H);
     } else {
-        rem_pass<T, LG, (1 << Ln::REM)>(v, buf, t, tw, sy);
+        const int p1 = (j >> 4) + (Q::H / 16) * (i >> 2);
+        return (j & 15) + 16 * (p1 + Q::HB * (i & 3));
     }
 }
 
-// Odd extension: v[r] = z[t + G r] holds for r < 8 on entry (z_0 = 0); the
-// values r >= 8 are -z[c G - t] for c = 16 - r (0 at c G - t = N), read from
-// the other threads' values through buf.
+// Whether that index is below G/2, the same for every thread.
+template <int LG>
+__host__ __device__ constexpr bool row_low(int i) {
+    using Q = Half<LG>;
+    return Q::H == 1 ? i < 8 : Q::HC == 1 ? i % Q::H < Q::H / 2 : (i & 3) < 2;
+}
+
+// Row transform, natural order to row_k order: v[r] = u[j + H r] on entry;
+// row: the row's G + 16 elements of shared memory (its values have been
+// read).
 template <typename T, int LG>
-__device__ __forceinline__ void reflect(Cplx<T> (&v)[16], CT<T>* buf, int t, const GSync& sy) {
-    using Ln = Len<LG>;
-    const int rb = t + (t >> 4);
+__device__ __forceinline__ void row_fwd(Cplx<T> (&v)[16], CT<T>* row, int j,
+                                        const CT<T>* __restrict__ tab) {
+    using Q = Half<LG>;
+    constexpr int H = Q::H, P2 = Q::P2, LIM = Q::RP;
+    dft_nat<T, 16>(v);
+    if constexpr (H > 1) {
 #pragma unroll
-    for (int r = 0; r < 8; ++r) stsl<T>(buf, rb + r * Ln::SG, v[r], Ln::LIM);
-    if (t == 0) stsl<T>(buf, sp(Ln::N), Cplx<T>{T(0), T(0)}, Ln::LIM);
-    sy.sync();
-    // sp(c G - t) = c sp(G) - (t + ceil(t / 16))
-    const int u = t + ((t + 15) >> 4);
+        for (int q = 1; q < 16; ++q) {
+            const Cplx<T> w = ldt<T>(tab + Q::T2, (q - 1) * H + j, Q::TABLE - Q::T2);
+            v[q] = cmul(v[q], w.x, w.y);
+        }
+        row_sync<LG>();   // every thread of the row has read its values
 #pragma unroll
-    for (int r = 8; r < 16; ++r) {
-        const Cplx<T> z = ldsl<T>(buf, (16 - r) * Ln::SG - u, Ln::LIM);
-        v[r] = Cplx<T>{-z.x, -z.y};
+        for (int q = 0; q < 16; ++q) sts_<T>(row, q * P2 + j, v[q], LIM);
+        row_sync<LG>();
+        if constexpr (Q::HC == 1) {
+#pragma unroll
+            for (int b = 0; b < 16 / H; ++b) {
+#pragma unroll
+                for (int e = 0; e < H; ++e)
+                    v[b * H + e] = lds_<T>(row, (j + H * b) * P2 + e, LIM);
+                dft_nat<T, H>(v + b * H);
+            }
+        } else {
+            constexpr int HB = Q::HB, NB = 16 / HB;
+            const int q = j & 15;
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                const int c = (j >> 4) + (H / 16) * b;   // j0
+#pragma unroll
+                for (int e = 0; e < HB; ++e)
+                    v[b * HB + e] = lds_<T>(row, q * P2 + c + 4 * e, LIM);
+                dft_nat<T, HB>(v + b * HB);
+#pragma unroll
+                for (int e = 0; e < HB; ++e) {
+                    if (e > 0) {
+                        const Cplx<T> w = ldt<T>(tab + Q::T3, e * 4 + c, Q::TABLE - Q::T3);
+                        v[b * HB + e] = cmul(v[b * HB + e], w.x, w.y);
+                    }
+                    sts_<T>(row, q * P2 + c + 4 * e, v[b * HB + e], LIM);   // in place
+                }
+            }
+            row_sync<LG>();
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const int p = (j >> 4) + (H / 16) * b;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[b * 4 + e] = lds_<T>(row, q * P2 + 4 * p + e, LIM);
+                dft_nat<T, 4>(v + b * 4);
+            }
+        }
     }
-    sy.sync();
 }
 
-// Rows a (and b when vb) of the right-hand side, elements j = t + G r,
-// r < 8 (j = 0 is the wall: 0): plane 0, plus plane 2 on rows with
-// row % part_py == 0, plus planes 1 and 3 at columns j % part_px == 0
-// (periods are powers of two: masks).
-// Every load of a row is issued before any sum.
-template <typename T, int G>
-__device__ __forceinline__ void load_rhs(const SolveParams<T>& P, const T* const (&in)[4], int ra,
-                                         int rb, bool va, bool vb, int t, Cplx<T> (&v)[16]) {
-    const long long n = (long long)(P.my + 1) * P.ld;
-    const size_t oa = (size_t)ra * P.ld + t, ob = (size_t)rb * P.ld + t;
-    const T* pa = in[0] + (va ? oa : 0);
-    const T* pb = in[0] + (vb ? ob : 0);
-    T a[8], b[8];
+// The same transform from row_k order to natural order: v[r] = V[j + H r]
+// on return.
+template <typename T, int LG>
+__device__ __forceinline__ void row_bwd(Cplx<T> (&v)[16], CT<T>* row, int j,
+                                        const CT<T>* __restrict__ tab) {
+    using Q = Half<LG>;
+    constexpr int H = Q::H, P2 = Q::P2, LIM = Q::RP;
+    if constexpr (H > 1) {
+        if constexpr (Q::HC == 1) {
+            row_sync<LG>();   // row_fwd's reads are done
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        const bool j0 = r == 0 && t == 0;
-        const bool ia = va && !j0 && QG_IN(oa + r * G, n, 63);
-        const bool ib = vb && !j0 && QG_IN(ob + r * G, n, 63);
-        a[r] = ia ? __ldg(pa + r * G) : T(0);
-        b[r] = ib ? __ldg(pb + r * G) : T(0);
+            for (int b = 0; b < 16 / H; ++b) {
+                dft_nat<T, H>(v + b * H);
+#pragma unroll
+                for (int e = 0; e < H; ++e)
+                    sts_<T>(row, (j + H * b) * P2 + e, v[b * H + e], LIM);
+            }
+        } else {
+            constexpr int HB = Q::HB, NB = 16 / HB;
+            const int q = j & 15;
+            row_sync<LG>();
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const int p = (j >> 4) + (H / 16) * b;
+                dft_nat<T, 4>(v + b * 4);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) sts_<T>(row, q * P2 + 4 * p + e, v[b * 4 + e], LIM);
+            }
+            row_sync<LG>();
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                const int c = (j >> 4) + (H / 16) * b;
+#pragma unroll
+                for (int e = 0; e < HB; ++e) {
+                    v[b * HB + e] = lds_<T>(row, q * P2 + c + 4 * e, LIM);
+                    if (e > 0) {
+                        const Cplx<T> w = ldt<T>(tab + Q::T3, e * 4 + c, Q::TABLE - Q::T3);
+                        v[b * HB + e] = cmul(v[b * HB + e], w.x, w.y);
+                    }
+                }
+                dft_nat<T, HB>(v + b * HB);
+#pragma unroll
+                for (int e = 0; e < HB; ++e)
+                    sts_<T>(row, q * P2 + c + 4 * e, v[b * HB + e], LIM);   // in place
+            }
+        }
+        row_sync<LG>();
+#pragma unroll
+        for (int q = 0; q < 16; ++q) {
+            v[q] = lds_<T>(row, q * P2 + j, LIM);
+            if (q > 0) {
+                const Cplx<T> w = ldt<T>(tab + Q::T2, (q - 1) * H + j, Q::TABLE - Q::T2);
+                v[q] = cmul(v[q], w.x, w.y);
+            }
+        }
     }
-    if (P.nin > 1) {
-        const bool ya = (ra & (P.part_py - 1)) == 0, yb = (rb & (P.part_py - 1)) == 0;
+    dft_nat<T, 16>(v);
+}
+
+// Columns j = t + G r (r < 8) and c G - t (c = 16 - r) of the right-hand side
+// rows ra and rb (existing: va, vb; planes ia, ib): plane 0, plus plane 2 on
+// rows with row % part_py == 0, plus planes 1 and 3 at columns with column %
+// part_px == 0.  The periods divide G, so one test of t serves every column.
+// Eight columns at a time: the loads of all their planes are in flight
+// together, within the register budget.
+template <typename T, int LG>
+__device__ __forceinline__ void load_rhs(const SolveParams<T>& P, const T* const (&ia)[4],
+                                         const T* const (&ib)[4], int ra, int rb, bool va, bool vb,
+                                         int t, Cplx<T> (&v)[16]) {
+    using Q = Half<LG>;
+    const int oa = (va ? ra : 0) * P.ld, ob = (vb ? rb : 0) * P.ld;
+    const bool cx = P.nin > 1 && (t & (P.part_px - 1)) == 0;
+    const bool ya = P.nin > 1 && va && (ra & (P.part_py - 1)) == 0;
+    const bool yb = P.nin > 1 && vb && (rb & (P.part_py - 1)) == 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        auto col = [&](int r) { return h == 0 ? t + Q::G * r : (8 - r) * Q::G - t; };
+        // not a wall (z_0, z_N)
+        auto ok = [&](int r) { return (t > 0 || r != 0) && QG_IN(col(r), P.mx, 63); };
+        T a[8], b[8];
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-            const int j = t + r * G;
-            const bool j0 = j == 0;
-            const bool ia = va && !j0 && QG_IN(oa + r * G, n, 63);
-            const bool ib = vb && !j0 && QG_IN(ob + r * G, n, 63);
-            const bool cx = (j & (P.part_px - 1)) == 0;
-            if (ia && ya) a[r] += __ldg(in[2] + oa + r * G);
-            if (ib && yb) b[r] += __ldg(in[2] + ob + r * G);
-            if (ia && cx) {
-                a[r] += __ldg(in[1] + oa + r * G);
-                if (ya) a[r] += __ldg(in[3] + oa + r * G);
+            a[r] = va && ok(r) ? __ldg(ia[0] + oa + col(r)) : T(0);
+            b[r] = vb && ok(r) ? __ldg(ib[0] + ob + col(r)) : T(0);
+        }
+        if (cx) {
+            T c[8], d[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                c[r] = va && ok(r) ? __ldg(ia[1] + oa + col(r)) : T(0);
+                d[r] = vb && ok(r) ? __ldg(ib[1] + ob + col(r)) : T(0);
             }
-            if (ib && cx) {
-                b[r] += __ldg(in[1] + ob + r * G);
-                if (yb) b[r] += __ldg(in[3] + ob + r * G);
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                a[r] += c[r];
+                b[r] += d[r];
             }
         }
+        auto add_seam = [&](const T* const (&in)[4], int o, T (&x)[8]) {
+            T c[8], d[8];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                c[r] = ok(r) ? __ldg(in[2] + o + col(r)) : T(0);
+                d[r] = cx && ok(r) ? __ldg(in[3] + o + col(r)) : T(0);
+            }
+#pragma unroll
+            for (int r = 0; r < 8; ++r) x[r] += c[r] + d[r];
+        };
+        if (ya) add_seam(ia, oa, a);
+        if (yb) add_seam(ib, ob, b);
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+            v[8 * h + r] = h == 0 ? Cplx<T>{a[r], b[r]} : Cplx<T>{-a[r], -b[r]};
     }
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = Cplx<T>{a[r], b[r]};
 }
 
-// Rows a and b of a scratch array (element j at column j - 1, j = 0: 0),
-// from row offsets oa, ob of arrays sa, sb with n elements.
-template <typename T, int G>
-__device__ __forceinline__ void load_rows(const T* sa, const T* sb, bool va, bool vb,
-                                          long long oa, long long ob, long long n, int t,
-                                          Cplx<T> (&v)[16]) {
-    const T* pa = sa + (va ? oa + t - 1 : 0);
-    const T* pb = sb + (vb ? ob + t - 1 : 0);
-    T a[8], b[8];
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        const bool j0 = r == 0 && t == 0;
-        const bool ia = va && !j0 && QG_IN(oa + t - 1 + r * G, n, 64);
-        const bool ib = vb && !j0 && QG_IN(ob + t - 1 + r * G, n, 64);
-        a[r] = ia ? __ldg(pa + r * G) : T(0);
-        b[r] = ib ? __ldg(pb + r * G) : T(0);
-    }
-#pragma unroll
-    for (int r = 0; r < 8; ++r) v[r] = Cplx<T>{a[r], b[r]};
+// 1/x for the normal range (an eigenvalue): the hardware's approximation
+// and Newton's iteration r (2 - x r) until the working precision.
+__device__ __forceinline__ float recip(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return fmaf(r, fmaf(-x, r, 1.0f), r);
+}
+__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+
+// Four consecutive values as vector stores (16-byte aligned).
+__device__ __forceinline__ void st4(float* p, float a, float b, float c, float d) {
+    *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
+}
+__device__ __forceinline__ void st4(double* p, double a, double b, double c, double d) {
+    *reinterpret_cast<double2*>(p) = make_double2(a, b);
+    *reinterpret_cast<double2*>(p + 2) = make_double2(c, d);
 }
 
-// Pairs per CTA of the passes that write transposed: `want`, fewer while
-// the CTA would exceed 1024 threads (FP32) or 512 (FP64, 128 registers per
-// thread) or 140 KB of shared memory.
-constexpr int kPpcX = 4, kPpcY = 4;   // x forward pass, y pass
-template <typename T>
-__host__ __device__ constexpr int ppc_for(int lg, int want) {
-    int p = want;
-    while (p > 1 && (((1 << lg) / 16) * p > (sizeof(T) == 4 ? 1024 : 512) ||
-                     (long long)p * buf_elems(1 << lg) * (long long)sizeof(T) * 2 > 140 * 1024))
-        p /= 2;
-    return p;
-}
-// Threads per CTA and the register budget: 64 per thread at 512 threads
-// and more, 80 below (FP32); 128 (FP64).
-template <typename T>
-__host__ __device__ constexpr int minb_for(int threads) {
-    const int regs = sizeof(T) == 8 ? 128 : (threads >= 512 ? 64 : 80);
-    const int b = 65536 / (threads * regs);
-    return b < 1 ? 1 : (b > 16 ? 16 : b);
+// Staging pitch in complex elements of the outputs of PPC pairs.
+__host__ __device__ constexpr int stage_pitch(int ppc) { return ppc == 1 ? 1 : ppc + 1; }
+__host__ __device__ constexpr int round32(int v) { return (v + 31) / 32 * 32; }
+
+// Threads of a CTA of PPC pairs, and its shared memory in complex elements:
+// the pairs' buffers (and a spare row when the last warp is not full), or
+// the staged outputs, never both at once.
+template <int LG, int PPC>
+__host__ __device__ constexpr int cta_threads() { return round32(Half<LG>::TP * PPC); }
+template <int LG, int PPC>
+__host__ __device__ constexpr int cta_elems(bool staged) {
+    const int buf = PPC * Half<LG>::BUF + (Half<LG>::TP * PPC % 32 ? Half<LG>::RP : 0);
+    const int stg = staged ? Half<LG>::N * stage_pitch(PPC) : 0;
+    return buf > stg ? buf : stg;
 }
 
-// Staging pitch (in T) of the transposed outputs of PPC pairs: 2 PPC
-// values per spectral index, padded against bank conflicts.
-__host__ __device__ constexpr int stage_pitch(int ppc) { return 2 * ppc + (ppc >= 4 ? 4 : 2); }
-
-// One pass of the solve for PPC sequence pairs per CTA (pair
-// blockIdx.x PPC + group, one group of G threads each).
-//   YP false, PH 0: rows ra, rb of the right-hand side -> tr[k][ra - 1, rb - 1];
-//   YP false, PH 2: rows ra, rb of work (element j at column j - 1) -> out;
-//   YP true:        x-modes ka, kb: rows of tr (element j at column j - 1),
-//                   forward transform, mode-space solve, inverse transform
-//                   -> work[l][ka - 1, kb - 1] (OPY 2: layers 0 and 1 of
-//                   x-mode ka).
-// The transposed outputs (tr, work) of the CTA's pairs are staged in shared
-// memory and written as runs of 2 PPC values per row.
-// One work item: PPC sequence pairs (pair blk PPC + group, one group of G
-// threads each) of phase PH, with P's arrays (a member's, for batches).
+// One pass of the solve for PPC sequence pairs (pair blk PPC + group, one
+// group of TP threads each; threads past the last group only meet the
+// barriers).  Pairs, one layer: two rows of the grid (x passes), two
+// positions (y pass); two layers: the two layers of a row or position.
 // Every thread of the CTA takes part.
 template <typename T, int OPY, int PH, int LG, int PPC>
 __device__ __forceinline__ void stream_item(const SolveParams<T>& P, int npairs, int blk,
                                             unsigned char* smem) {
-    using Ln = Len<LG>;
-    constexpr bool YP = PH == 1;
-    constexpr int G = Ln::G;
-    const int grp = PPC == 1 ? 0 : (int)threadIdx.x / G;
-    const int t = (int)threadIdx.x - grp * G;
+    using Q = Half<LG>;
+    constexpr int G = Q::G, H = Q::H, N = Q::N;
+    const int grp = PPC == 1 && Q::TP % 32 == 0 ? 0 : (int)threadIdx.x / Q::TP;
+    const int tt = (int)threadIdx.x - grp * Q::TP;
+    const bool act = grp < PPC;
+    const int s = tt / H, j = tt - s * H;      // the thread's row and place in it
+    const bool tpass = act && tt <= G / 2;     // takes part in the radix-16 pass
     const int pair0 = blk * PPC, pair = pair0 + grp;
-    const bool vp = pair < npairs;
-    CT<T>* buf = reinterpret_cast<CT<T>*>(smem) + grp * Ln::LIM;
-    const GSync sy{1 + grp, G, PPC == 1};
-    int layer = 0, ra, rb;
-    bool vb;
-    if (YP) {
-        if (OPY == 2) {
-            ra = rb = 1 + pair;
-            vb = vp;
-        } else {
-            ra = 1 + 2 * pair;
-            rb = ra + 1;
-            vb = vp && rb <= P.mx - 1;
-        }
-    } else {
-        const int ppl = P.my / 2;
-        layer = pair0 / ppl;       // ppl is a multiple of PPC: one layer per CTA
-        ra = 1 + 2 * (pair - layer * ppl);
-        rb = ra + 1;
-        vb = vp && rb <= P.my - 1;
-    }
-    const CT<T>* tw = YP ? P.pty : P.ptx;
-    // the layer's arrays, selected without indexing (an indexed parameter
-    // array would be copied to local memory)
-    const bool l1 = layer != 0;
-    const T* const in[4] = {l1 ? P.in[1][0] : P.in[0][0], l1 ? P.in[1][1] : P.in[0][1],
-                            l1 ? P.in[1][2] : P.in[0][2], l1 ? P.in[1][3] : P.in[0][3]};
-    T* const trl = l1 ? P.tr[1] : P.tr[0];
-    T* const workl = l1 ? P.work[1] : P.work[0];
-    T* const outl = l1 ? P.out[1] : P.out[0];
+    const bool vp = act && pair < npairs;
+    CT<T>* buf = reinterpret_cast<CT<T>*>(smem) + (act ? grp : 0) * Q::BUF;
+    // (threads past the last group run the row stages on a spare row)
+    CT<T>* row = act ? buf + s * Q::RP : reinterpret_cast<CT<T>*>(smem) + PPC * Q::BUF;
+    const CT<T>* tab = PH == 1 ? P.hty : P.htx;
+    // scratch arrays, in complex units of two interleaved sequences
+    CT<T>* tr = reinterpret_cast<CT<T>*>(P.tr[0]);
+    CT<T>* wk = reinterpret_cast<CT<T>*>(P.work[0] + P.ld);   // from row 1 of the array on
+    const long long ntr = (long long)(OPY == 2 ? P.mx : P.mx / 2) * P.ld_tr;
+    const long long nwk = (long long)(OPY == 2 ? P.my - 1 : P.my / 2) * P.ld;
+    (void)ntr;
+    (void)nwk;
 
     Cplx<T> v[16];
-    if (YP) {
-        const long long n = (long long)(P.mx + 1) * P.ld_tr;
-        load_rows<T, G>(P.tr[0], P.tr[OPY == 2 ? 1 : 0], vp, vb, (long long)ra * P.ld_tr,
-                        (long long)rb * P.ld_tr, n, t, v);
-    } else if (PH == 0) {
-        load_rhs<T, G>(P, in, ra, rb, vp, vb, t, v);
-    } else {
-        const long long n = (long long)(P.my + 1) * P.ld;
-        load_rows<T, G>(workl, workl, vp, vb, (long long)ra * P.ld,
-                        (long long)rb * P.ld, n, t, v);
-    }
-    reflect<T, LG>(v, buf, t, sy);
-    fft16s<T, LG>(v, buf, t, tw, sy);
-
-    if (YP) {
-        // mode-space solve of the modes l = t + G s, s < 8 (l = 0: the wall)
-        const T lxa = QG_IN(ra, P.mx + 1, 66) ? __ldg(P.lamx + ra) : T(1);
-        const T lxb = QG_IN(rb, P.mx + 1, 66) ? __ldg(P.lamx + rb) : T(1);
-        const T* ly_t = P.lamy + t;
+    if constexpr (PH == 2) {
+        // row s of the inverse x pass: modes s + 16 k, k = j + H r; k >= G/2
+        // are the negated modes 16 - s + 16 (G - 1 - k)
+        const CT<T>* src = wk + (vp ? (size_t)pair * P.ld : 0);
 #pragma unroll
-        for (int s = 0; s < 8; ++s) {
-            const T Fa = T(-0.5) * v[s].y, Fb = T(0.5) * v[s].x;
-            T x = T(0), y = T(0);
-            if (vp && (s > 0 || t > 0) && QG_IN(t + s * G, P.my + 1, 67)) {
-                const T ly = __ldg(ly_t + s * G);
-                if (OPY == 1) {
-                    x = Fa * (P.scale / (lxa + ly));
-                    if (vb) y = Fb * (P.scale / (lxb + ly));
-                } else {
-                    const T q1 = P.scale * Fa, q2 = P.scale * Fb;
-                    const T al = P.Ro * (lxa + ly);
-                    const T den = al * (al - P.f1 - P.f2);
-                    x = (al * q1 - P.f2 * q1 - P.f1 * q2) / den;
-                    y = (al * q2 - P.f2 * q1 - P.f1 * q2) / den;
+        for (int r = 0; r < 16; ++r) {
+            const int k = j + H * r;
+            int pos, zero;
+            if (r < 8) {
+                pos = s * (G / 2) + k;
+                zero = s == 0 && k == 0;
+            } else {
+                pos = s == 0 ? G - k : (16 - s) * (G / 2) + G - 1 - k;
+                zero = s == 0 && k == G / 2;
+            }
+            CT<T> x;
+            x.x = x.y = T(0);
+            if (vp && !zero && QG_IN((long long)pair * P.ld + pos, nwk, 64)) x = src[pos];
+            v[r] = r < 8 ? Cplx<T>{x.x, x.y} : Cplx<T>{-x.x, -x.y};
+        }
+        row_fwd<T, LG>(v, row, j, tab);
+        row_sync<LG>();
+        if (act) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) sts_<T>(row, row_k<LG>(j, i), v[i], Q::RP);
+        }
+    } else {
+        if (tpass) {
+            if constexpr (PH == 0) {
+                const int ra = OPY == 2 ? 1 + pair : 1 + 2 * pair, rb = OPY == 2 ? ra : ra + 1;
+                load_rhs<T, LG>(P, P.in[0], P.in[OPY == 2 ? 1 : 0], ra, rb, vp,
+                                vp && rb <= P.my - 1, tt, v);
+            } else {
+                const CT<T>* src = tr + (vp ? (size_t)pair * P.ld_tr : 0) - 1;
+#pragma unroll
+                for (int r = 0; r < 16; ++r) {
+                    const int n = r < 8 ? tt + G * r : (16 - r) * G - tt;
+                    CT<T> x;
+                    x.x = x.y = T(0);
+                    if (vp && (tt > 0 || (r & 7) != 0) &&
+                        QG_IN((long long)pair * P.ld_tr + n - 1, ntr, 65))
+                        x = src[n];
+                    v[r] = r < 8 ? Cplx<T>{x.x, x.y} : Cplx<T>{-x.x, -x.y};
                 }
             }
-            v[s] = Cplx<T>{x, y};
-        }
-        reflect<T, LG>(v, buf, t, sy);
-        fft16s<T, LG>(v, buf, t, tw, sy);
-    }
-
-    // F(a)_k = -Im Z_k / 2, F(b)_k = Re Z_k / 2 for k = t + G s < N
-    if constexpr (PH == 2) {
-        const long long nw = (long long)(P.my + 1) * P.ld;
-        T* oa = outl + (size_t)ra * P.ld + t;
-        T* ob = outl + (size_t)rb * P.ld + t;
-#pragma unroll
-        for (int s = 0; s < 8; ++s) {
-            const T fa = T(-0.5) * v[s].y, fb = T(0.5) * v[s].x;
-            const bool k0 = s == 0 && t == 0;
-            if (vp && QG_IN((long long)ra * P.ld + t + s * G, nw, 70)) oa[s * G] = k0 ? T(0) : fa;
-            if (vb && QG_IN((long long)rb * P.ld + t + s * G, nw, 70)) ob[s * G] = k0 ? T(0) : fb;
-        }
-    } else {
-        // transposed outputs: stage [k][2 group + (0: a, 1: b)], then write runs
-        constexpr int SP = stage_pitch(PPC), W = 2 * PPC;
-        T* stg = reinterpret_cast<T*>(smem);
-        __syncthreads();   // every group is done with its FFT buffer
-#pragma unroll
-        for (int s = 0; s < 8; ++s) {
-            CT<T> o;
-            o.x = T(-0.5) * v[s].y;
-            o.y = T(0.5) * v[s].x;
-            const int i = (t + s * G) * SP + 2 * grp;
-            if (QG_IN(i + 1, (long long)PPC * Ln::LIM * 2, 71))
-                *reinterpret_cast<CT<T>*>(stg + i) = o;
+            pass_fwd<T, LG>(v, buf, tt, tab);
         }
         __syncthreads();
-        // thread e of the CTA writes column q = e mod W of rows
-        // k = e / W + i G / 2 (G PPC threads cover G / 2 rows per step)
-        const int q = (int)threadIdx.x % W, k0 = (int)threadIdx.x / W;
-        constexpr int KSTEP = G / 2, ITER = Ln::N / KSTEP;
-        if (YP) {
-            // work[l][c], l = 1..my-1; OPY 1: c = 2 pair0 + q; OPY 2: layer
-            // q % 2 at column pair0 + q / 2
+#pragma unroll
+        for (int r = 0; r < 16; ++r) v[r] = lds_<T>(row, j + H * r, Q::RP);
+        row_fwd<T, LG>(v, row, j, tab);
+    }
+
+    if constexpr (PH == 1) {
+        // mode-space solve of the modes l = s + 16 k, their images included
+        // (the eigenvalues of l and 2 my - l are the same); the walls l = 0
+        // and my stay 0
+        auto mode = [&](int pos) { return pos / (P.mx / 16) + 16 * (pos % (P.mx / 16)); };
+        const int ka = OPY == 2 ? mode(pair) : mode(2 * pair);
+        const int kb = OPY == 2 ? ka : mode(2 * pair + 1);
+        const bool ok = vp && QG_IN(ka, P.mx + 1, 66) && QG_IN(kb, P.mx + 1, 66);
+        const T lxa = ok ? __ldg(P.lamx + ka) : T(1), lxb = ok ? __ldg(P.lamx + kb) : T(1);
+        const T* ly_s = P.lamyr + s * G;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const int k = row_k<LG>(j, i);
+            const bool wall = s == 0 && (k == 0 || k == G / 2);
+            const bool in = act && !wall && QG_IN(s * G + k, 9 * G, 67);
+            const T ly = in ? __ldg(ly_s + k) : T(1);
+            // the pair's 2 F are -Im Z and Re Z
+            const T Fa = -v[i].y, Fb = v[i].x;
+            T x, y;
+            if (OPY == 1) {
+                x = Fa * (P.scale * recip(lxa + ly));
+                y = Fb * (P.scale * recip(lxb + ly));
+            } else {
+                const T q1 = P.scale * Fa, q2 = P.scale * Fb;
+                const T al = P.Ro * (lxa + ly);
+                const T den = al * (al - P.f1 - P.f2);
+                x = (al * q1 - P.f2 * q1 - P.f1 * q2) / den;
+                y = (al * q2 - P.f2 * q1 - P.f1 * q2) / den;
+            }
+            v[i] = in ? Cplx<T>{x, y} : Cplx<T>{T(0), T(0)};
+        }
+        row_bwd<T, LG>(v, row, j, tab);
+        row_sync<LG>();
+        if (act) {
+#pragma unroll
+            for (int r = 0; r < 16; ++r) sts_<T>(row, j + H * r, v[r], Q::RP);
+        }
+    }
+    if constexpr (PH >= 1) {
+        __syncthreads();
+        if (tpass) pass_bwd<T, LG>(v, buf, tt, tab);
+    }
+
+    // 2 F(a)_k = -Im Z_k, 2 F(b)_k = Re Z_k (P.scale holds the 2^-4)
+    if constexpr (PH == 2) {
+        if (tpass) {
+            const int ra = OPY == 2 ? 1 + pair : 1 + 2 * pair, rb = OPY == 2 ? ra : ra + 1;
+            const bool vb = vp && rb <= P.my - 1;
             const long long nw = (long long)(P.my + 1) * P.ld;
-            const int c = OPY == 1 ? 2 * pair0 + q : pair0 + (q >> 1);
-            T* dst = (OPY == 1 || !(q & 1) ? P.work[0] : P.work[1]) + c;
-            const bool vc = c <= P.mx - 2;
-#pragma unroll 4
-            for (int i = 0; i < ITER; ++i) {
-                const int k = k0 + i * KSTEP;
-                if (k > 0 && vc && QG_IN((long long)k * P.ld + c, nw, 72))
-                    dst[(size_t)k * P.ld] = stg[k * SP + q];
+            (void)nw;
+            T* oa = P.out[0] + (vp ? (size_t)ra * P.ld : 0);
+            T* ob = P.out[OPY == 2 ? 1 : 0] + (vp ? (size_t)rb * P.ld : 0);
+            // (column 0 and the wall row my are zero: out may be the array
+            // that held the scratch values)
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const bool second = r >= 8;
+                const int n = second ? (16 - r) * G - tt : tt + G * r;
+                const bool wall = tt == 0 && (r & 7) == 0;      // n = 0 or N
+                if (second && !wall && (tt == 0 || tt == G / 2)) continue;   // seen at r < 8
+                const T sg = second ? T(-1) : T(1);
+                const T fa = wall ? T(0) : -sg * v[r].y, fb = wall || !vb ? T(0) : sg * v[r].x;
+                if (vp && QG_IN((long long)ra * P.ld + n, nw, 70)) oa[n] = fa;
+                if (vp && QG_IN((long long)rb * P.ld + n, nw, 70)) ob[n] = fb;
+            }
+        }
+    } else {
+        constexpr int SP = stage_pitch(PPC);
+        CT<T>* stg = reinterpret_cast<CT<T>*>(smem);
+        constexpr int SLIM = cta_elems<LG, PPC>(true);
+        __syncthreads();   // every group is done with its buffer
+        if constexpr (PH == 0) {
+            // modes s + 16 k by position
+            if (act) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    const int k = row_k<LG>(j, i);
+                    const bool low = row_low<LG>(i);
+                    if (!low && (s == 0 || s == 8)) continue;   // images of the low half
+                    const int pos = low ? s * (G / 2) + k : (16 - s) * (G / 2) + G - 1 - k;
+                    const T sg = low ? T(1) : T(-1);
+                    Cplx<T> o{-sg * v[i].y, sg * v[i].x};
+                    if (pos == 0) o = Cplx<T>{T(0), T(0)};      // the wall mode
+                    sts_<T>(stg, pos * SP + grp, o, SLIM);
+                }
             }
         } else {
-            // tr[k][c], k = 1..mx-1, c = 2 (pair0 - layer ppl) + q
-            const long long ntr = (long long)(P.mx + 1) * P.ld_tr;
-            const int c = 2 * (pair0 - layer * (P.my / 2)) + q;
-            T* dst = trl + c;
-            const bool vc = c <= P.my - 2;
+            if (tpass) {
+#pragma unroll
+                for (int r = 0; r < 16; ++r) {
+                    const bool second = r >= 8;
+                    const int n = second ? (16 - r) * G - tt : tt + G * r;
+                    if (tt == 0 && (r & 7) == 0) continue;
+                    if (second && (tt == 0 || tt == G / 2)) continue;
+                    const T sg = second ? T(-1) : T(1);
+                    sts_<T>(stg, n * SP + grp, Cplx<T>{-sg * v[r].y, sg * v[r].x}, SLIM);
+                }
+            }
+        }
+        __syncthreads();
+        // thread e writes for pair g = e mod PPC the items e / PPC + i STEP
+        constexpr int BT = cta_threads<LG, PPC>(), STEP = BT / PPC;
+        static_assert(BT % PPC == 0, "");
+        const int g = (int)threadIdx.x % PPC, q0 = (int)threadIdx.x / PPC;
+        const int ldo = PH == 0 ? P.ld_tr : P.ld;
+        if (pair0 + g < npairs) {
+            if constexpr (OPY == 1) {
+                // 2 x 2 blocks: positions 2 q, 2 q + 1 (x forward) or rows
+                // 2 q + 1, 2 q + 2 (y) of a pair, transposed into a run of 4
+                // values
+                constexpr int ITEMS = N / 2, ITER = (ITEMS + STEP - 1) / STEP;
+                const CT<T>* src = stg + (PH == 0 ? 2 * q0 : 2 * q0 + 1) * SP + g;
+                long long o = (long long)q0 * ldo + 2 * (pair0 + g);
+                CT<T>* dst = PH == 0 ? tr : wk;
 #pragma unroll 4
-            for (int i = 0; i < ITER; ++i) {
-                const int k = k0 + i * KSTEP;
-                if (k > 0 && vc && QG_IN((long long)k * P.ld_tr + c, ntr, 69))
-                    dst[(size_t)k * P.ld_tr] = stg[k * SP + q];
+                for (int i = 0; i < ITER; ++i) {
+                    const int q = q0 + i * STEP;
+                    if (q < ITEMS && QG_IN((2 * q + 1) * SP + g, SLIM, 61) &&
+                        QG_IN(o + 1, PH == 0 ? ntr : nwk, PH == 0 ? 69 : 72)) {
+                        const CT<T> c0 = src[2 * i * STEP * SP];
+                        CT<T> c1;
+                        c1.x = c1.y = T(0);      // (row N is the wall)
+                        if (PH == 0 || q < ITEMS - 1) c1 = src[(2 * i * STEP + 1) * SP];
+                        st4(reinterpret_cast<T*>(dst + o), c0.x, c1.x, c0.y, c1.y);
+                    }
+                    o += (long long)STEP * ldo;
+                }
+            } else {
+                // [position][row][layer] (x forward), [row][position][layer] (y)
+                constexpr int ITER = (N + STEP - 1) / STEP;
+                const CT<T>* src = stg + q0 * SP + g;
+                long long o = (long long)(PH == 0 ? q0 : q0 - 1) * ldo + pair0 + g;
+                CT<T>* dst = PH == 0 ? tr : wk;
+#pragma unroll 4
+                for (int i = 0; i < ITER; ++i) {
+                    const int q = q0 + i * STEP;
+                    if (q < N && (PH == 0 || q > 0) && QG_IN(q * SP + g, SLIM, 61) &&
+                        QG_IN(o, PH == 0 ? ntr : nwk, PH == 0 ? 69 : 72))
+                        dst[o] = src[i * STEP * SP];
+                    o += (long long)STEP * ldo;
+                }
             }
         }
     }
+}
+
+// Registers per thread the CTA shapes are budgeted for: FP32 72 (three CTAs
+// of 288 threads per SM; at 96, two, the passes of the 2048 x 4096 grid took
+// 29, 59 and 20 us instead of 22, 41 and 20), FP64 as many as it takes.
+template <typename T>
+__host__ __device__ constexpr int minb_for(int threads, int regs32 = 72) {
+    const int regs = sizeof(T) == 8 ? 160 : regs32;
+    const int b = 65536 / (round32(threads) * regs);
+    return b < 1 ? 1 : (b > 16 ? 16 : b);
 }
 
 // One launch per pass.  Batches (ensembles, one layer): member
 // blockIdx.x / cpm takes CTAs blockIdx.x mod cpm, with its arrays from
 // P.batch.
 template <typename T, int OPY, int PH, int LG, int PPC>
-__global__ void __launch_bounds__(Len<LG>::G * PPC, minb_for<T>(Len<LG>::G * PPC))
+__global__ void __launch_bounds__(cta_threads<LG, PPC>(), minb_for<T>(cta_threads<LG, PPC>()))
 stream_kernel(SolveParams<T> Pin, int npairs, int cpm) {
     extern __shared__ __align__(16) unsigned char smem[];
     SolveParams<T> P = Pin;
@@ -527,6 +666,13 @@ stream_kernel(SolveParams<T> Pin, int npairs, int cpm) {
     stream_item<T, OPY, PH, LG, PPC>(P, npairs, blk, smem);
 }
 
+// Pairs per y item of the work queue (twice as many per x item, half as
+// long) and its CTA size.
+__host__ __device__ constexpr int queue_ppc(int lgx) { return lgx <= 9 ? 4 : lgx == 10 ? 4 : 2; }
+__host__ __device__ constexpr int queue_threads(int lgx) {
+    return round32(9 * (1 << (lgx + 1)) / 256 * queue_ppc(lgx));
+}
+
 // Batched solve of an ensemble group in one launch (one layer, y length
 // twice the x length): a work queue over the items of the three passes of
 // every member, claimed in order from the counter q[0] (pass by pass,
@@ -536,8 +682,7 @@ stream_kernel(SolveParams<T> Pin, int npairs, int cpm) {
 // no later item, so the wait ends without any co-residency.  A wait that
 // runs out sets the member's error flag and the item is counted done
 // unprocessed.  The last CTA to leave resets the counters for the next
-// launch.  The CTA has BT threads: BT / G_x pairs per x item, BT / G_y per
-// y item.
+// launch.
 constexpr int kQueueSpin = 1 << 22;
 
 __device__ __forceinline__ bool wait_done(const unsigned* c, unsigned want, int limit) {
@@ -549,13 +694,13 @@ __device__ __forceinline__ bool wait_done(const unsigned* c, unsigned want, int 
     return false;
 }
 
-template <typename T, int LGX, int BT>
-__global__ void __launch_bounds__(BT, minb_for<T>(BT))
+template <typename T, int LGX>
+__global__ void __launch_bounds__(queue_threads(LGX), minb_for<T>(queue_threads(LGX), 96))
 stream_queue_kernel(SolveParams<T> P) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_item;
     constexpr int LGY = LGX + 1;
-    constexpr int PX = BT / Len<LGX>::G, PY = BT / Len<LGY>::G;
+    constexpr int PX = 2 * queue_ppc(LGX), PY = queue_ppc(LGX);
     unsigned* q = P.bar;
     const int nb = P.nbatch;
     const int rows = P.my / 2, cols = P.mx / 2;
@@ -615,20 +760,16 @@ stream_queue_kernel(SolveParams<T> P) {
     }
 }
 
-// Lengths 2^LG of the engine: L = 512 .. 16384 (FP32), .. 8192 (FP64).
-constexpr int kMinLg = 9, kMaxLg = 14;
+// Lengths 2^LG of the engine: L = 256 .. 16384 (FP32), .. 8192 (FP64).
+constexpr int kMinLg = 8, kMaxLg = 14;
 
-template <typename T, int OPY, int PH, int LG>
-cudaError_t launch_pass(const SolveParams<T>& P, int npairs, cudaStream_t s) {
-    constexpr int PPC = PH == 2 ? 1 : ppc_for<T>(LG, PH == 0 ? kPpcX : kPpcY);
-    constexpr int G = Len<LG>::G;
+template <typename T, int OPY, int PH, int LG, int PPC>
+cudaError_t launch_ppc(const SolveParams<T>& P, int npairs, cudaStream_t s) {
     const int cpm = (npairs + PPC - 1) / PPC;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cpm * (P.batch ? P.nbatch : 1));
-    cfg.blockDim = dim3(G * PPC);
-    const size_t fft_bytes = (size_t)PPC * Len<LG>::LIM * sizeof(CT<T>);
-    const size_t stg_bytes = PH == 2 ? 0 : (size_t)Len<LG>::N * stage_pitch(PPC) * sizeof(T);
-    cfg.dynamicSmemBytes = fft_bytes > stg_bytes ? fft_bytes : stg_bytes;
+    cfg.blockDim = dim3(cta_threads<LG, PPC>());
+    cfg.dynamicSmemBytes = (size_t)cta_elems<LG, PPC>(PH != 2) * sizeof(CT<T>);
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -638,16 +779,68 @@ cudaError_t launch_pass(const SolveParams<T>& P, int npairs, cudaStream_t s) {
     cfg.attrs = P.no_pdl ? nullptr : at;
     cfg.numAttrs = P.no_pdl ? 0 : 1;
     auto k = stream_kernel<T, OPY, PH, LG, PPC>;
-    cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k),
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)cfg.dynamicSmemBytes);
+    int per = 0, nsm = 0;
+    cudaError_t e = launch_shape(reinterpret_cast<const void*>(k), (int)cfg.blockDim.x,
+                                 cfg.dynamicSmemBytes, &per, &nsm);
     if (e != cudaSuccess) return e;
     return cudaLaunchKernelEx(&cfg, k, P, npairs, cpm);
+}
+
+// Pairs per CTA, of 1, 2, .. ppc_max (CTAs of at most 288 threads, FP32 at
+// LG = 12 576): the number that leaves the fullest SM the fewest warps.  More
+// pairs fill the CTA's last warp and write longer runs, so a tie takes more
+// pairs (the inverse x pass writes whole rows either way: fewer, in FP32);
+// with few warps on an SM the pass is bound by latency, and fewer pairs are
+// taken for up to an eighth more warps.  Measured in whole FP32 steps at
+// l = 0 (us; pairs in the three passes): 512 x 1024 51.8 with (4, 2, 2),
+// 55.4 with (4, 1, 1); 1024 x 2048 79.9 with (4, 4, 1), 93.1 with (4, 2, 1);
+// 512 x 2048 64.4 with (4, 1, 4), 69.8 with (8, 1, 4); 2048 x 4096 291 with
+// (2, 1, 2), 298 with (4, 1, 1); FP64 512 x 1024 575 with (4, 2, 4), 661
+// with (4, 2, 1).
+template <typename T>
+__host__ __device__ constexpr int ppc_max(int lg) {
+    return lg <= 10 ? 8 : lg == 11 ? 4 : lg == 12 ? (sizeof(T) == 4 ? 4 : 2) : 1;
+}
+template <typename T>
+int pick_ppc(int ph, int lg, int npairs, int batch, int nsm) {
+    const int tp = 9 * (1 << lg) / 256;
+    int best = 1, cost = 0;
+    for (int c = 1; c <= ppc_max<T>(lg); c *= 2) {
+        const int ctas = (npairs + c - 1) / c * batch;
+        const int w = (ctas + nsm - 1) / nsm * (round32(tp * c) / 32);
+        const bool keep_tie = ph == 2 && sizeof(T) == 4;
+        if (c == 1 || w < cost || (w == cost && !keep_tie)) {
+            if (c > 1 && cost <= 16 && 8 * cost <= 9 * w) continue;
+            best = c;
+            cost = w;
+        }
+    }
+    return best;
+}
+template <typename T, int OPY, int PH, int LG>
+cudaError_t launch_pass(const SolveParams<T>& P, int npairs, cudaStream_t s) {
+    int dev = 0, nsm = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int c = pick_ppc<T>(PH, LG, npairs, P.batch ? P.nbatch : 1, nsm);
+    constexpr int M = ppc_max<T>(LG);
+    if constexpr (M >= 8) {
+        if (c == 8) return launch_ppc<T, OPY, PH, LG, 8>(P, npairs, s);
+    }
+    if constexpr (M >= 4) {
+        if (c == 4) return launch_ppc<T, OPY, PH, LG, 4>(P, npairs, s);
+    }
+    if constexpr (M >= 2) {
+        if (c == 2) return launch_ppc<T, OPY, PH, LG, 2>(P, npairs, s);
+    }
+    return launch_ppc<T, OPY, PH, LG, 1>(P, npairs, s);
 }
 
 template <typename T, int OPY, int PH>
 cudaError_t launch_lg(const SolveParams<T>& P, int lg, int npairs, cudaStream_t s) {
     switch (lg) {
+        case 8: return launch_pass<T, OPY, PH, 8>(P, npairs, s);
         case 9: return launch_pass<T, OPY, PH, 9>(P, npairs, s);
         case 10: return launch_pass<T, OPY, PH, 10>(P, npairs, s);
         case 11: return launch_pass<T, OPY, PH, 11>(P, npairs, s);
@@ -663,41 +856,24 @@ cudaError_t launch_lg(const SolveParams<T>& P, int lg, int npairs, cudaStream_t 
 template <typename T, int OPY>
 cudaError_t launch_all(const SolveParams<T>& P, cudaStream_t s) {
     const int lgx = ilog2(2 * P.mx), lgy = ilog2(2 * P.my);
-    const int rows = (P.my / 2) * P.layers;
-    const int cols = OPY == 2 ? P.mx - 1 : P.mx / 2;
+    const int rows = OPY == 2 ? P.my - 1 : P.my / 2;
+    const int cols = OPY == 2 ? P.mx : P.mx / 2;
     cudaError_t e = launch_lg<T, OPY, 0>(P, lgx, rows, s);
     if (e == cudaSuccess) e = launch_lg<T, OPY, 1>(P, lgy, cols, s);
     if (e == cudaSuccess) e = launch_lg<T, OPY, 2>(P, lgx, rows, s);
     return e;
 }
 
-// The work-queue launch of a batch: the CTA size and pairs per item.
-template <typename T>
-constexpr int queue_threads(int lgx) {
-    const int gy = (1 << (lgx + 1)) / 16;
-    const int maxt = sizeof(T) == 4 ? 1024 : 512;
-    return 4 * gy < maxt ? 4 * gy : maxt;
-}
-
 template <typename T, int LGX>
 cudaError_t launch_queue_lg(const SolveParams<T>& P, cudaStream_t s) {
-    constexpr int BT = queue_threads<T>(LGX);
-    constexpr int PX = BT / Len<LGX>::G, PY = BT / Len<LGX + 1>::G;
-    auto k = stream_queue_kernel<T, LGX, BT>;
-    size_t sm = (size_t)PX * Len<LGX>::LIM * sizeof(CT<T>);
-    const size_t smy = (size_t)PY * Len<LGX + 1>::LIM * sizeof(CT<T>);
-    const size_t stx = (size_t)Len<LGX>::N * stage_pitch(PX) * sizeof(T);
-    const size_t sty = (size_t)Len<LGX + 1>::N * stage_pitch(PY) * sizeof(T);
-    for (size_t v : {smy, stx, sty}) sm = v > sm ? v : sm;
-    cudaError_t e = cudaFuncSetAttribute(reinterpret_cast<const void*>(k),
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    constexpr int BT = queue_threads(LGX);
+    constexpr int PX = 2 * queue_ppc(LGX), PY = queue_ppc(LGX);
+    auto k = stream_queue_kernel<T, LGX>;
+    constexpr int ex = cta_elems<LGX, PX>(true), ey = cta_elems<LGX + 1, PY>(true);
+    const size_t sm = (size_t)(ex > ey ? ex : ey) * sizeof(CT<T>);
+    int nsm = 0, per = 0;
+    cudaError_t e = launch_shape(reinterpret_cast<const void*>(k), BT, sm, &per, &nsm);
     if (e != cudaSuccess) return e;
-    int dev = 0, nsm = 0, per = 0;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-        return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, BT, sm)) != cudaSuccess)
-        return e;
     if (per < 1) return cudaErrorInvalidConfiguration;
     const int rows = P.my / 2, cols = P.mx / 2;
     const int total = P.nbatch * (2 * ((rows + PX - 1) / PX) + (cols + PY - 1) / PY);
@@ -718,28 +894,69 @@ cudaError_t launch_queue_lg(const SolveParams<T>& P, cudaStream_t s) {
 
 }  // namespace
 
-// Batches of one-layer grids with my = 2 mx and 2 mx = 2^9 .. 2^11 run as
+// Batches of one-layer grids with my = 2 mx and 2 mx = 2^8 .. 2^11 run as
 // one work-queue launch; other batches as three launches.
 bool stream_queue_ok(int mx, int my, int layers) {
     if (layers != 1 || my != 2 * mx || !is_pow2(mx)) return false;
     const int lx = ilog2(2 * mx);
-    return lx >= 9 && lx <= 11;
+    return lx >= 8 && lx <= 11;
 }
 
 bool stream_supports(int mx, int my, size_t esz) {
     if (!is_pow2(mx) || !is_pow2(my)) return false;
     const int lx = ilog2(2 * mx), ly = ilog2(2 * my);
     const int hi = esz == 4 ? kMaxLg : kMaxLg - 1;
+    // (128 x 128 and less are left to the engines of one launch)
+    if (lx == kMinLg && ly == kMinLg) return false;
     return lx >= kMinLg && ly >= kMinLg && lx <= hi && ly <= hi;
 }
 
+size_t half_table_size(int L) {
+    const int G = L / 16, H = G / 16;
+    return (size_t)8 * (G / 2 + 2) + 15 * H + (H > 16 ? H : 0);
+}
+
+void half_table(int L, double* re, double* im) {
+    const int G = L / 16, H = G / 16, PT = G / 2 + 2;
+    const double pi = 3.14159265358979323846;
+    auto put = [&](size_t i, long long num, long long den) {   // e^{-2 pi i num/den}
+        const double a = -2.0 * pi * (double)(num % den) / (double)den;
+        re[i] = std::cos(a);
+        im[i] = std::sin(a);
+    };
+    for (int s = 1; s <= 8; ++s)
+        for (int t = 0; t < PT; ++t) put((size_t)(s - 1) * PT + t, (long long)t * s, L);
+    const size_t t2 = (size_t)8 * PT, t3 = t2 + 15 * (size_t)H;
+    for (int q = 1; q < 16; ++q)
+        for (int j = 0; j < H; ++j) put(t2 + (size_t)(q - 1) * H + j, (long long)q * j, G);
+    if (H > 16)
+        for (int p = 0; p < H / 4; ++p)
+            for (int c = 0; c < 4; ++c) put(t3 + 4 * p + c, (long long)p * c, H);
+}
+
+void half_lam(int M, const double* lam, double* out) {
+    const int G = M / 8;
+    for (int s = 0; s <= 8; ++s)
+        for (int k = 0; k < G; ++k) {
+            const int m = s + 16 * k;
+            out[(size_t)s * G + k] = lam[m <= M ? m : 2 * M - m];
+        }
+}
+
 template <typename T>
-cudaError_t launch_solve_stream(const SolveParams<T>& P, cudaStream_t s) {
-    if (!stream_supports(P.mx, P.my, sizeof(T)) || !P.ptx || !P.pty ||
-        (P.batch && (P.layers != 1 || P.nbatch < 1)))
+cudaError_t launch_solve_stream(const SolveParams<T>& Pin, cudaStream_t s) {
+    if (!stream_supports(Pin.mx, Pin.my, sizeof(T)) || !Pin.htx || !Pin.hty || !Pin.lamyr ||
+        (Pin.batch && (Pin.layers != 1 || Pin.nbatch < 1)))
         return cudaErrorInvalidValue;
+    // two layers: the scratch rows of both layers lie in one run from work[0]
+    // (tr[0]), so the output may not share them
+    if (Pin.layers == 2 && (Pin.out[0] == Pin.work[0] || Pin.out[1] == Pin.work[1]))
+        return cudaErrorInvalidValue;
+    SolveParams<T> P = Pin;
+    P.scale *= T(1) / T(16);   // the passes leave 2 F (exact)
     if (P.batch && stream_queue_ok(P.mx, P.my, P.layers) && P.bar) {
         switch (ilog2(2 * P.mx)) {
+            case 8: return launch_queue_lg<T, 8>(P, s);
             case 9: return launch_queue_lg<T, 9>(P, s);
             case 10: return launch_queue_lg<T, 10>(P, s);
             default: return launch_queue_lg<T, 11>(P, s);
