@@ -288,7 +288,8 @@ qg_status qg_set_solver(qg_handle h, qg_solver kind, int32_t cycles);
  * transforms (radix-16 passes with the values in registers, only the half
  * that the odd symmetry leaves), several sequence pairs per CTA and three
  * launches (one per pass), for elliptic grids of 128 to 8192 intervals a side (4096 in
- * FP64) above 128 x 128; 0:
+ * FP64) above 128 x 128; 42: the sine sums with one output per thread, three
+ * launches, for elliptic grids of at most 256 intervals a side; 0:
  * the multigrid solver (qg_set_solver).  These are
  * implementations of the same sine-transform solve of Section 4.3, equal to
  * rounding.  No device work.  Errors: QG_ERR_ARG.                          */
@@ -302,6 +303,9 @@ qg_status qg_solve_engine(qg_handle h, int32_t* engine);
  * FP32 handles take 128, 64 or 32 rows with 8 rows per thread (16 at
  * l = 4), or 64 or 32 rows with 4 rows per thread at l <= 2 (shorter CTAs:
  * a smaller last wave); FP64 and two-layer handles keep 64 and 128 rows.
+ * One-layer handles of both types also take 8 rows (16 at l = 4) with 1 row
+ * per thread: tiles 16 columns wide with one node per thread, for grids
+ * whose other tiles would leave most of the GPU idle.
  * QG_FINE_ROWS=<rows> or <rows>x<rows per thread> forces an offered tile.
  * Ensemble members keep the default.  The tiles give the same results to
  * rounding.  No device work.  Errors: QG_ERR_ARG.                          */

@@ -54,6 +54,8 @@ struct LevelTables {
     void* htx = nullptr;                         // engine 50: twiddles for L = 2 mx and
     void* hty = nullptr;                         //   2 my, and the y eigenvalues in the
     void* lamyr = nullptr;                       //   order of its rows
+    void* dsx = nullptr;                         // engine 42: sine tables of mx and my
+    void* dsy = nullptr;
     void* mtab = nullptr;  // matrix engine (FP32, one layer): sine matrices and 1/lambda
     void* tctab = nullptr; // engine 41: split sine matrices (shared-memory image), 1/lambda
 };
@@ -317,29 +319,6 @@ qg_status get_pass_table(qg_ctx* h, int L, int rad, void** out) {
     return QG_OK;
 }
 
-// The twiddle table of engine 50 for length L (half_table).
-qg_status get_half_table(qg_ctx* h, int L, void** out) {
-    const int key = -(L * 64 + 63);   // shares the twiddle cache with the pass tables
-    auto it = h->twcache.find(key);
-    if (it != h->twcache.end()) {
-        *out = it->second;
-        return QG_OK;
-    }
-    const size_t n = half_table_size(L);
-    std::vector<double> re(n), im(n), v(2 * n);
-    half_table(L, re.data(), im.data());
-    for (size_t k = 0; k < n; ++k) {
-        v[2 * k] = re[k];
-        v[2 * k + 1] = im[k];
-    }
-    void* d = nullptr;
-    qg_status s = upload_real(h, &d, v);
-    if (s != QG_OK) return s;
-    h->twcache[key] = d;
-    *out = d;
-    return QG_OK;
-}
-
 // Eigenvalue and twiddle tables of grid level `lv` (Eq. ialpha without Ro).
 qg_status get_level(qg_ctx* h, int lv, const LevelTables** out) {
     auto it = h->tables.find(lv);
@@ -388,12 +367,32 @@ qg_status get_level(qg_ctx* h, int lv, const LevelTables** out) {
     for (int l = 1; l < t.my; ++l) ly[l] = (2.0 * std::cos(pi * l / t.my) - 2.0) / (t.dyc * t.dyc);
     s = upload_real(h, &t.lamx, lx);
     if (s == QG_OK) s = upload_real(h, &t.lamy, ly);
+    // the tables of engines 50 and 42, one upload each (their parts start on
+    // 16 bytes: even counts)
     if (s == QG_OK && stream_supports(t.mx, t.my, h->esz)) {
-        s = get_half_table(h, 2 * t.mx, &t.htx);
-        if (s == QG_OK) s = get_half_table(h, 2 * t.my, &t.hty);
-        std::vector<double> lr((size_t)9 * (t.my / 8));
-        half_lam(t.my, ly.data(), lr.data());
-        if (s == QG_OK) s = upload_real(h, &t.lamyr, lr);
+        const size_t nx = half_table_size(2 * t.mx), ny = half_table_size(2 * t.my);
+        const size_t nl = (size_t)9 * (t.my / 8), nm = nx > ny ? nx : ny;
+        std::vector<double> v(2 * (nx + ny) + nl), re(nm), im(nm);
+        for (int d = 0; d < 2; ++d) {
+            half_table(2 * (d ? t.my : t.mx), re.data(), im.data());
+            double* o = v.data() + (d ? 2 * nx : 0);
+            for (size_t k = 0; k < (d ? ny : nx); ++k) {
+                o[2 * k] = re[k];
+                o[2 * k + 1] = im[k];
+            }
+        }
+        half_lam(t.my, ly.data(), v.data() + 2 * (nx + ny));
+        s = upload_real(h, &t.htx, v);
+        t.hty = static_cast<char*>(t.htx) + 2 * nx * h->esz;
+        t.lamyr = static_cast<char*>(t.htx) + 2 * (nx + ny) * h->esz;
+    }
+    if (s == QG_OK && !h->member && dense_supports(t.mx, t.my)) {
+        const size_t nx = (size_t)t.mx * t.mx / 2, ny = (size_t)t.my * t.my / 2;
+        std::vector<double> v(nx + ny);
+        dense_table(t.mx, v.data());
+        dense_table(t.my, v.data() + nx);
+        s = upload_real(h, &t.dsx, v);
+        t.dsy = static_cast<char*>(t.dsx) + nx * h->esz;
     }
     if (s != QG_OK) return s;
     h->tables[lv] = t;
@@ -551,7 +550,7 @@ qg_status solve_level(qg_ctx* h, const LevelTables& t, const void* in, void* tr,
     P.nin = nparts;
     P.part_px = P.part_py = 1;
     if (nparts > 1) {
-        P.part_px = fine_part_period_x(h->levels);
+        P.part_px = fine_part_period_x(h->levels, h->fine_ry);
         P.part_py = fine_part_period_y(h->levels, h->fine_rows);
     }
     P.ld = t.ldc;
@@ -566,6 +565,8 @@ qg_status solve_level(qg_ctx* h, const LevelTables& t, const void* in, void* tr,
     P.htx = static_cast<const C*>(t.htx);
     P.hty = static_cast<const C*>(t.hty);
     P.lamyr = static_cast<const T*>(t.lamyr);
+    P.dsx = static_cast<const T*>(t.dsx);
+    P.dsy = static_cast<const T*>(t.dsy);
     P.lamx = static_cast<const T*>(t.lamx);
     P.lamy = static_cast<const T*>(t.lamy);
     P.scale = (T)((2.0 / t.mx) * (2.0 / t.my));
@@ -611,7 +612,7 @@ qg_status solve_level(qg_ctx* h, const LevelTables& t, const void* in, void* tr,
 // (nx, ny, levels, layers, dtype) for the process and, when the environment
 // variable QG_TUNE_CACHE names a file, in that file (one line
 // "nx ny levels layers esz engine rows ry" per entry; ensemble groups add
-// lines "group mx my dx dy members esz engine").  QG_SOLVE_ENGINE=4|16|32|33|34|40|41|50
+// lines "group mx my dx dy members esz engine").  QG_SOLVE_ENGINE=4|16|32|33|34|40|41|42|50
 // forces a choice where that engine supports the grid.  Other grids use the
 // size rule.
 
@@ -628,6 +629,7 @@ bool engine_ok(const qg_ctx* h, const LevelTables* t, size_t esz, int e) {
     if (e == kMatrixEngine) return t->mtab && mtx_supports(t->mx, t->my, esz, h->layers);
     if (e == kTcEngine) return t->tctab && tc_supports(t->mx, t->my, esz, h->layers);
     if (e == kStreamEngine) return solve_engine_supports(t->mx, t->my, esz, e) && t->htx;
+    if (e == kDenseEngine) return t->dsx && t->dsy;
     return solve_engine_supports(t->mx, t->my, esz, e) && (!is_warp_engine(e) || t->ptx[e - 32]);
 }
 
@@ -672,7 +674,7 @@ std::map<GroupKey, int> g_batch_tune;
 
 bool known_engine(int e) {
     return e == 4 || e == 16 || is_warp_engine(e) || e == kMatrixEngine || e == kTcEngine ||
-           e == kStreamEngine;
+           e == kStreamEngine || e == kDenseEngine;
 }
 
 // (called with g_tune_mutex held)
@@ -784,7 +786,8 @@ qg_status autotune_solve(qg_ctx* h) {
     using Tile = std::pair<int, int>;
     std::vector<Tile> tiles{{h->fine_rows, h->fine_ry}};
     if (!h->member)
-        for (Tile c : {Tile{64, h->fine_ry}, Tile{32, h->fine_ry}, Tile{64, 4}, Tile{32, 4}})
+        for (Tile c : {Tile{64, h->fine_ry}, Tile{32, h->fine_ry}, Tile{64, 4}, Tile{32, 4},
+                       Tile{node_tile_rows(h->levels), 1}})
             if (c != tiles[0] && fine_rows_supported(h->esz, h->layers, h->levels, c.first, c.second))
                 tiles.push_back(c);
     // QG_FINE_ROWS=<rows> or <rows>x<rows per thread> forces an offered tile
@@ -805,7 +808,10 @@ qg_status autotune_solve(qg_ctx* h) {
     };
     const bool forced_rows = forced.first != 0;
     if (forced_rows) QG_TRY_S(set_tile(forced));
-    if (const char* force = std::getenv("QG_SOLVE_ENGINE")) {
+    // a forced engine that does not take the grid leaves the choice to the
+    // transforms (engines 4 to 34 and 50)
+    const char* force = std::getenv("QG_SOLVE_ENGINE");
+    if (force) {
         const int e = std::atoi(force);
         if (engine_ok(h, t, sizeof(T), e)) {
             h->solve_engine = e;
@@ -820,7 +826,8 @@ qg_status autotune_solve(qg_ctx* h) {
         auto it = g_tune_cache.find(key);
         const Tile cached{it == g_tune_cache.end() ? 0 : it->second.rows,
                           it == g_tune_cache.end() ? 0 : it->second.ry};
-        if (it != g_tune_cache.end() &&
+        if (it != g_tune_cache.end() && engine_ok(h, t, sizeof(T), it->second.engine) &&
+            !(force && it->second.engine == kDenseEngine) &&
             std::find(tiles.begin(), tiles.end(), cached) != tiles.end()) {
             h->solve_engine = it->second.engine;
             if (!forced_rows) QG_TRY_S(set_tile(cached));
@@ -835,14 +842,15 @@ qg_status autotune_solve(qg_ctx* h) {
     const float t40 = time_steps<T>(h, kMatrixEngine);
     const float t50 = time_steps<T>(h, kStreamEngine);
     const float t41 = time_steps<T>(h, kTcEngine);
+    const float t42 = force ? 1e30f : time_steps<T>(h, kDenseEngine);
     // a candidate that cannot run on this grid is a tuning result, not an error
     h->latched = QG_OK;
     (void)cudaGetLastError();
     drop_graph(h);
-    const float tt[8] = {t4, t16, t32, t33, t34, t40, t50, t41};
-    const int ee[8] = {4, 16, 32, 33, 34, kMatrixEngine, kStreamEngine, kTcEngine};
+    const float tt[9] = {t4, t16, t32, t33, t34, t40, t50, t41, t42};
+    const int ee[9] = {4,  16, 32, 33, 34, kMatrixEngine, kStreamEngine, kTcEngine, kDenseEngine};
     int best = 0;
-    for (int k = 1; k < 8; ++k)
+    for (int k = 1; k < 9; ++k)
         if (tt[k] < tt[best]) best = k;
     if (tt[best] >= 1e29f) return fail(h, QG_ERR_CUDA);
     h->solve_engine = ee[best];
@@ -865,6 +873,7 @@ qg_status autotune_solve(qg_ctx* h) {
     }
     // the timing steps ran on the handle's buffers: return them to rest
     QG_TRY_S(rest_buffers(h, h->stream));
+    if (force) return QG_OK;   // (a choice among some of the engines is not kept)
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     const TuneVal v{h->solve_engine, h->fine_rows, h->fine_ry};
     g_tune_cache[key] = v;
@@ -1817,8 +1826,8 @@ qg_status qg_bounds_check_result(int32_t* site) {
     }
     int first = 0;
     for (int v : {bounds_site_fused(), bounds_site_solve32(), bounds_site_stencil(),
-                  bounds_site_mtx(), bounds_site_stream(), bounds_site_tc(), qg::bounds_site_mg(),
-                  qg::bounds_site_diag(), qg::bounds_site_adjoint()}) {
+                  bounds_site_mtx(), bounds_site_stream(), bounds_site_node(), bounds_site_dense(),
+                  bounds_site_tc(), qg::bounds_site_mg(), qg::bounds_site_diag(), qg::bounds_site_adjoint()}) {
         if (v < 0) return QG_ERR_CUDA;
         if (!first) first = v;
     }
@@ -2388,7 +2397,7 @@ qg_status ensemble_tables(qg_ensemble e) {
                 } else {
                     for (int q = 0; q < 4; ++q) M.in[q] = plane<T>(h->part, h->plane_c, q);
                     M.nin = 4;
-                    M.part_px = fine_part_period_x(h->levels);
+                    M.part_px = fine_part_period_x(h->levels, h->fine_ry);
                     M.part_py = fine_part_period_y(h->levels, h->fine_rows);
                     M.out = static_cast<T*>(h->cpsi);
                 }

@@ -686,6 +686,9 @@ cudaError_t launch_fine_fused(const FusedParams<T>& p, const FineMaps& m, int le
                               cudaStream_t s, bool two_layer, int rows, int ry) {
     constexpr int R0 = Rows<T>::value;
     const int ry0 = levels >= 4 ? 16 : 8;
+    if (ry == 1)
+        return two_layer || rows != node_tile_rows(levels) ? cudaErrorInvalidValue
+                                                           : launch_fine_node<T>(p, levels, s);
     if (two_layer) {   // l >= 1 only: the other layer's psi comes from the elliptic grid
         if (rows != R0 || ry != ry0) return cudaErrorInvalidValue;
         switch (levels) {
@@ -758,11 +761,12 @@ int fine_rows_per_thread(int levels) { return levels >= 4 ? 16 : 8; }
 bool fine_rows_supported(size_t esz, int layers, int levels, int rows, int ry) {
     const int ry0 = fine_rows_per_thread(levels);
     if (rows == (int)fine_tile_rows(esz) && ry == ry0) return true;
+    if (ry == 1) return layers == 1 && rows == node_tile_rows(levels);
     if (esz != 4 || layers != 1) return false;
     if (ry == ry0) return rows == 64 || rows == 32;
     return ry == 4 && levels <= 2 && (rows == 64 || rows == 32);
 }
-int fine_part_period_x(int levels) { return TX >> levels; }
+int fine_part_period_x(int levels, int ry) { return (ry == 1 ? node_tile_cols() : TX) >> levels; }
 int fine_part_period_y(int levels, int rows) { return rows >> levels; }
 int fine_halo_cols() { return SWX; }
 int fine_block_cols() { return TX; }

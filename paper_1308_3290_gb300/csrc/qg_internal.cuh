@@ -75,6 +75,8 @@ struct SolveParams {
     const typename Cx<T>::type* htx;   // engine 50: half_table(2 mx) and
     const typename Cx<T>::type* hty;   //   half_table(2 my)
     const T* lamyr;                     // engine 50: lamy in its rows' order (half_lam)
+    const T* dsx;                       // engine 42: dense_table(mx) and
+    const T* dsy;                       //   dense_table(my)
     const T* lamx;                      // (2 cos(pi k/mx) - 2)/dx^2, k = 0..mx
     const T* lamy;                      // (2 cos(pi l/my) - 2)/dy^2, l = 0..my
     T scale, Ro, f1, f2;
@@ -131,8 +133,17 @@ template <typename T>
 cudaError_t launch_solve_stream(const SolveParams<T>& P, cudaStream_t s);
 // batched engine-50 solves that run as one work-queue launch
 bool stream_queue_ok(int mx, int my, int layers);
+// engine 42: the sine sums one output per thread, three launches
+// (solve_dense.cu); grids of at most 256 intervals a side, no batches.  Its
+// table for N intervals: sin(pi n k / N) at [(n - 1) N + k], n = 1..N/2
+constexpr int kDenseEngine = 42;
+bool dense_supports(int mx, int my);
+void dense_table(int N, double* out);
+template <typename T>
+cudaError_t launch_solve_dense(const SolveParams<T>& P, cudaStream_t s);
 // the kernels one solve of an engine launches (a batch of members: `batch`)
 inline int solve_launches(int engine, int mx = 0, int my = 0, bool batch = false) {
+    if (engine == kDenseEngine) return 3;
     if (engine != kStreamEngine) return 1;
     return batch && stream_queue_ok(mx, my, 1) ? 1 : 3;
 }
@@ -278,7 +289,13 @@ size_t fine_tile_rows(size_t esz);   // default fine rows per CTA
 int ensemble_tile_rows(size_t esz);  // fine rows per CTA of ensemble members
 int fine_rows_per_thread(int levels);   // default rows a thread sweeps
 bool fine_rows_supported(size_t esz, int layers, int levels, int rows, int ry);  // tuned pairs
-int fine_part_period_x(int levels);  // coarse columns between tile edges
+int fine_part_period_x(int levels, int ry);  // coarse columns between tile edges
+// The stage with one node per thread (fused_node.cu; one layer): tiles of
+// node_tile_cols x node_tile_rows nodes, named by one row per thread.
+template <typename T>
+cudaError_t launch_fine_node(const FusedParams<T>& p, int levels, cudaStream_t s);
+int node_tile_rows(int levels);
+int node_tile_cols();
 int fine_part_period_y(int levels, int rows);  // coarse rows between CTA edges
 int fine_halo_cols();                // columns of a halo box
 int fine_block_cols();               // columns of an interior box
@@ -366,6 +383,8 @@ int bounds_site_solve32();
 int bounds_site_stencil();
 int bounds_site_mtx();
 int bounds_site_stream();
+int bounds_site_node();
+int bounds_site_dense();
 
 // Copies between the dense exchange layout and the padded node layout.
 cudaError_t copy_in(void* padded, int ld, const void* dense, int nxm1,

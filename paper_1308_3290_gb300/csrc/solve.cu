@@ -407,6 +407,7 @@ size_t solve_smem_bytes(int mx, int my, size_t esz, int engine) {
 
 bool solve_engine_supports(int mx, int my, size_t esz, int engine) {
     if (engine == kStreamEngine) return stream_supports(mx, my, esz);
+    if (engine == kDenseEngine) return dense_supports(mx, my);
     if (is_warp_engine(engine)) {
         const int rad = warp_engine_radix(engine);
         return solve32_supports(mx, my, rad, esz) &&
@@ -435,6 +436,7 @@ cudaError_t launch_solve(const SolveParams<T>& P, int engine, cudaStream_t s) {
         return cudaErrorInvalidValue;
     if (is_warp_engine(engine)) return launch_solve32<T>(P, warp_engine_radix(engine), s);
     if (engine == kStreamEngine) return launch_solve_stream<T>(P, s);
+    if (engine == kDenseEngine) return launch_solve_dense<T>(P, s);
     if (P.batch) return cudaErrorInvalidValue;   // batches: warp-group engines only
     return engine == 4 ? launch_engine<T, 4>(P, s) : launch_engine<T, 16>(P, s);
 }
