@@ -121,6 +121,7 @@ struct qg_ctx {
     cudaGraphExec_t gexec = nullptr;
     qg_status latched = QG_OK;
     std::vector<void*> allocs;
+    cudaMemPool_t pool = nullptr;  // scratch of the stand-alone calls (scratch_alloc)
     size_t alloc_bytes = 0;        // device bytes held through dev_alloc
     // per-kernel timing (bench instrumentation): events recorded in the graph
     bool timing = false;
@@ -621,6 +622,9 @@ int engine_rule(int mx, int my) { return (long)mx * my >= (1L << 21) ? 16 : 4; }
 int engine_for(qg_ctx* h, int mx, int my) {
     const LevelTables* t = nullptr;
     if (get_level(h, h->levels, &t) == QG_OK && t->mx == mx && t->my == my) return h->solve_engine;
+    // other levels are not timed: the half-length transforms where they take
+    // the grid (2048 x 4096 FP32: 77 us, radix 16 over 240 us)
+    if (stream_supports(mx, my, h->esz)) return kStreamEngine;
     return engine_rule(mx, my);
 }
 
@@ -1333,6 +1337,7 @@ qg_status qg_destroy(qg_handle h) {
     tape_release(h);
     drop_graph(h);
     for (void* p : h->allocs) cudaFree(p);
+    if (h->pool) cudaMemPoolDestroy(h->pool);
     for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
     if (h->hout) cudaFreeHost(h->hout);
     if (h->cap) cudaStreamDestroy(h->cap);
@@ -1498,6 +1503,25 @@ qg_status qg_set_forcing(qg_handle h, const void* forcing) {
     return QG_OK;
 }
 
+// Scratch of one stand-alone call, on the handle's stream, from a pool of the
+// handle's own: the default pool gives its memory back to the driver at
+// every synchronisation, and taking it again cost 200 us a call.  The pool
+// holds no more than the largest call used and goes with the handle.
+static cudaError_t scratch_alloc(qg_ctx* h, void** p, size_t bytes) {
+    if (!h->pool) {
+        cudaMemPoolProps pp = {};
+        pp.allocType = cudaMemAllocationTypePinned;
+        pp.location.type = cudaMemLocationTypeDevice;
+        cudaError_t e = cudaGetDevice(&pp.location.id);
+        if (e == cudaSuccess) e = cudaMemPoolCreate(&h->pool, &pp);
+        uint64_t keep = UINT64_MAX;
+        if (e == cudaSuccess)
+            e = cudaMemPoolSetAttribute(h->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaMallocFromPoolAsync(p, bytes, h->pool, h->stream);
+}
+
 qg_status qg_poisson_solve(qg_handle h, const void* rhs, void* psi, int level) {
     NvtxRange nvtx_range("qg_poisson_solve");
     if (!h || !rhs || !psi || level < 0 || level > h->levels) return QG_ERR_ARG;
@@ -1517,7 +1541,7 @@ qg_status qg_poisson_solve(qg_handle h, const void* rhs, void* psi, int level) {
     const size_t apart = h->layers == 2 ? pl * h->layers * h->esz : 0;
     const size_t bytes = pl * h->layers * h->esz + part2 + apart;
     void* buf = nullptr;
-    QG_TRY(cudaMallocAsync(&buf, bytes, h->stream));
+    QG_TRY(scratch_alloc(h, &buf, bytes));
     void* tbuf = static_cast<char*>(buf) + pl * h->layers * h->esz;
     cudaError_t e = cudaMemsetAsync(buf, 0, bytes, h->stream);
     const size_t dense = (size_t)(t->mx - 1) * (t->my - 1) * h->esz;
@@ -1554,10 +1578,26 @@ static qg_status transfer(qg_handle h, const void* src, void* dst, int levels, b
     if (h->latched != QG_OK) return qg_last_error(h);
     const int mx = h->nx >> levels, my = h->ny >> levels, ldc = padded_ld(mx);
     const size_t bf = h->plane_f * h->esz, bc = (size_t)(my + 1) * ldc * h->esz;
+    // device buffers that do not overlap: straight from one to the other
+    const size_t nf = (size_t)(h->nx - 1) * (h->ny - 1) * h->esz;
+    const size_t nc = (size_t)(mx - 1) * (my - 1) * h->esz;
+    const char *s0 = static_cast<const char*>(src), *d0 = static_cast<const char*>(dst);
+    const size_t ns = down ? nf : nc, nd = down ? nc : nf;
+    if (on_device(src) && on_device(dst) && (s0 + ns <= d0 || d0 + nd <= s0)) {
+        auto go = [&](auto t) {
+            using T = decltype(t);
+            const T* a = static_cast<const T*>(src);
+            T* b = static_cast<T*>(dst);
+            return down ? launch_restrict_dense<T>(a, b, h->nx, h->ny, levels, h->stream)
+                        : launch_prolong_dense<T>(a, b, h->nx, h->ny, levels, h->stream);
+        };
+        QG_TRY(h->dtype == QG_F64 ? go(double()) : go(float()));
+        return QG_OK;
+    }
     void* f = nullptr;
     void* c = nullptr;
-    QG_TRY(cudaMallocAsync(&f, bf, h->stream));
-    cudaError_t e = cudaMallocAsync(&c, bc, h->stream);
+    QG_TRY(scratch_alloc(h, &f, bf));
+    cudaError_t e = scratch_alloc(h, &c, bc);
     if (e == cudaSuccess) e = cudaMemsetAsync(f, 0, bf, h->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c, 0, bc, h->stream);
     if (down) {

@@ -160,6 +160,14 @@ template <typename T>
 cudaError_t launch_prolong(const T* coarse, int ldc, T* fine, int ldf,
                            int nx, int ny, int levels, cudaStream_t s);
 
+// The same on fields in the exchange layout (device memory, not overlapping).
+template <typename T>
+cudaError_t launch_restrict_dense(const T* fine, T* coarse, int nx, int ny, int levels,
+                                  cudaStream_t s);
+template <typename T>
+cudaError_t launch_prolong_dense(const T* coarse, T* fine, int nx, int ny, int levels,
+                                 cudaStream_t s);
+
 // Constants of one fine-grid stage of the one-layer model.
 template <typename T>
 struct StageParams {
@@ -386,6 +394,8 @@ int bounds_site_stream();
 int bounds_site_node();
 int bounds_site_dense();
 
+// Whether ptr is device memory (not host or managed).
+bool on_device(const void* ptr);
 // Copies between the dense exchange layout and the padded node layout.
 cudaError_t copy_in(void* padded, int ld, const void* dense, int nxm1,
                     int nym1, size_t esz, cudaStream_t s);

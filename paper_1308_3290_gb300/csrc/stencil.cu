@@ -121,7 +121,9 @@ __global__ void restrict_kernel(const T* __restrict__ fine, int ldf,
 }
 
 // P^l as bilinear interpolation from the coarse nodes around each fine node.
-template <typename T>
+// DENSE: both fields in the exchange layout, coarse and fine pointing where
+// node (0, 0) would lie: the walls are not stored and count as zero.
+template <typename T, bool DENSE>
 __global__ void prolong_kernel(const T* __restrict__ coarse, int ldc,
                                T* __restrict__ fine, int ldf, int nx, int ny,
                                int levels) {
@@ -133,12 +135,16 @@ __global__ void prolong_kernel(const T* __restrict__ coarse, int ldc,
     const T a = T(i & (f - 1)) / T(f);
     const T b = T(j & (f - 1)) / T(f);
     const T* C = coarse + (size_t)J * ldc + I;
-    // the coarse grid has (ny >> levels) + 1 rows of pitch ldc
-    if (!QG_IN((long long)(J + 1) * ldc + I + 1, (long long)((ny >> levels) + 1) * ldc, 43))
-        return;
-    const T v = (T(1) - a) * (T(1) - b) * C[0] + a * (T(1) - b) * C[1] +
-                (T(1) - a) * b * C[ldc] + a * b * C[ldc + 1];
-    if (QG_IN((long long)j * ldf + i, (long long)(ny + 1) * ldf, 44))
+    const int mx = nx >> levels, my = ny >> levels;
+    // the coarse grid has my + 1 rows of pitch ldc
+    if (!DENSE && !QG_IN((long long)(J + 1) * ldc + I + 1, (long long)(my + 1) * ldc, 43)) return;
+    auto at = [&](int di, int dj) {
+        if (DENSE && !(I + di >= 1 && I + di < mx && J + dj >= 1 && J + dj < my)) return T(0);
+        return C[(size_t)dj * ldc + di];
+    };
+    const T v = (T(1) - a) * (T(1) - b) * at(0, 0) + a * (T(1) - b) * at(1, 0) +
+                (T(1) - a) * b * at(0, 1) + a * b * at(1, 1);
+    if (DENSE || QG_IN((long long)j * ldf + i, (long long)(ny + 1) * ldf, 44))
         fine[(size_t)j * ldf + i] = v;
 }
 
@@ -176,11 +182,31 @@ cudaError_t launch_restrict(const T* fine, int ldf, T* coarse, int ldc, int mx,
 }
 
 template <typename T>
+cudaError_t launch_restrict_dense(const T* fine, T* coarse, int nx, int ny, int levels,
+                                  cudaStream_t s) {
+    // interior nodes only are read and written, so the exchange layout is a
+    // padded one of pitch nx - 1 whose node (1, 1) is the first value
+    const int mx = nx >> levels, my = ny >> levels, ldf = nx - 1, ldc = mx - 1;
+    return launch_restrict<T>(fine - (ldf + 1), ldf, coarse - (ldc + 1), ldc, mx, my, levels, s);
+}
+
+template <typename T>
 cudaError_t launch_prolong(const T* coarse, int ldc, T* fine, int ldf, int nx,
                            int ny, int levels, cudaStream_t s) {
     const dim3 block(32, 8);
     const dim3 grid((nx - 1 + 31) / 32, (ny - 1 + 7) / 8);
-    prolong_kernel<T><<<grid, block, 0, s>>>(coarse, ldc, fine, ldf, nx, ny, levels);
+    prolong_kernel<T, false><<<grid, block, 0, s>>>(coarse, ldc, fine, ldf, nx, ny, levels);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_prolong_dense(const T* coarse, T* fine, int nx, int ny, int levels,
+                                 cudaStream_t s) {
+    const int ldc = (nx >> levels) - 1, ldf = nx - 1;
+    const dim3 block(32, 8);
+    const dim3 grid((nx - 1 + 31) / 32, (ny - 1 + 7) / 8);
+    prolong_kernel<T, true><<<grid, block, 0, s>>>(coarse - (ldc + 1), ldc, fine - (ldf + 1), ldf,
+                                                   nx, ny, levels);
     return cudaGetLastError();
 }
 
@@ -369,38 +395,47 @@ cudaError_t launch_mean_out(T* dense, const double* acc, int ldacc, double scale
 // dense (nym1 rows of nxm1) <-> padded interior.  The dense side (often
 // pinned host memory reached over the C2C link) moves in 16-byte vectors
 // of the flat array when it is 16-byte aligned, the padded side element by
-// element; both are row-contiguous, so both sides coalesce.
-template <typename W>
-__global__ void repack_kernel(W* __restrict__ dst, const W* __restrict__ src, int nxm1, int nym1,
-                              int ld, int to_padded) {
-    constexpr int V = 16 / sizeof(W);
-    const long n = (long)nxm1 * nym1;
-    const W* dense_r = to_padded ? src : nullptr;
-    W* dense_w = to_padded ? nullptr : dst;
-    const bool vec = ((reinterpret_cast<uintptr_t>(to_padded ? (const void*)src : (const void*)dst)
-                       & 15) == 0);
-    const long nv = vec ? n / V : 0;
-    auto pad = [&](long e) { const int j = (int)(e / nxm1); return (size_t)(j + 1) * ld + (e - (long)j * nxm1) + 1; };
-    for (long g = (long)blockIdx.x * blockDim.x + threadIdx.x; g < nv;
-         g += (long)gridDim.x * blockDim.x) {
+// element; both are row-contiguous, so both sides coalesce.  One 32-bit
+// division per vector (a field has less than 2^27 values; with a 64-bit one
+// per element the index arithmetic was the kernel's time).
+template <typename W, bool TO_PADDED>
+__global__ void __launch_bounds__(256)
+repack_kernel(W* __restrict__ dst, const W* __restrict__ src, unsigned nxm1, unsigned nym1, int ld) {
+    constexpr unsigned V = 16 / sizeof(W);
+    const unsigned n = nxm1 * nym1, stride = gridDim.x * blockDim.x;
+    const unsigned t0 = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool vec = (reinterpret_cast<uintptr_t>(TO_PADDED ? (const void*)src : (const void*)dst) & 15) == 0;
+    const unsigned nv = vec ? n / V : 0;
+#pragma unroll 2
+    for (unsigned g = t0; g < nv; g += stride) {
         W v[V];
-        if (to_padded) {
-            const uint4 u = reinterpret_cast<const uint4*>(dense_r)[g];
+        unsigned j = g * V / nxm1, i = g * V - j * nxm1;
+        size_t o = (size_t)(j + 1) * ld + i + 1;
+        if (TO_PADDED) {
+            const uint4 u = reinterpret_cast<const uint4*>(src)[g];
             memcpy(v, &u, 16);
+        }
 #pragma unroll
-            for (int k = 0; k < V; ++k) dst[pad(g * V + k)] = v[k];
-        } else {
-#pragma unroll
-            for (int k = 0; k < V; ++k) v[k] = src[pad(g * V + k)];
+        for (unsigned k = 0; k < V; ++k) {
+            if (TO_PADDED) dst[o] = v[k];
+            else v[k] = src[o];
+            ++o;
+            if (++i == nxm1) {
+                i = 0;
+                o += ld - nxm1;
+            }
+        }
+        if (!TO_PADDED) {
             uint4 u;
             memcpy(&u, v, 16);
-            reinterpret_cast<uint4*>(dense_w)[g] = u;
+            reinterpret_cast<uint4*>(dst)[g] = u;
         }
     }
-    for (long e = nv * V + (long)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-         e += (long)gridDim.x * blockDim.x) {
-        if (to_padded) dst[pad(e)] = src[e];
-        else dst[e] = src[pad(e)];
+    for (unsigned e = nv * V + t0; e < n; e += stride) {
+        const unsigned j = e / nxm1;
+        const size_t o = (size_t)(j + 1) * ld + (e - j * nxm1) + 1;
+        if (TO_PADDED) dst[o] = src[e];
+        else dst[e] = src[o];
     }
 }
 
@@ -424,16 +459,28 @@ static cudaError_t repack(void* dst, const void* src, int nxm1, int nym1, int ld
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const long n = (long)nxm1 * nym1;
     long blocks = (n + 255) / 256;
-    if (blocks > 16L * nsm) blocks = 16L * nsm;
-    if (esz == 8)
-        repack_kernel<double><<<(int)blocks, 256, 0, s>>>(static_cast<double*>(dst),
-                                                          static_cast<const double*>(src), nxm1,
-                                                          nym1, ld, to_padded ? 1 : 0);
-    else
-        repack_kernel<float><<<(int)blocks, 256, 0, s>>>(static_cast<float*>(dst),
-                                                         static_cast<const float*>(src), nxm1,
-                                                         nym1, ld, to_padded ? 1 : 0);
+    if (blocks > 8L * nsm) blocks = 8L * nsm;
+    auto go = [&](auto w) {
+        using W = decltype(w);
+        if (to_padded)
+            repack_kernel<W, true><<<(int)blocks, 256, 0, s>>>(static_cast<W*>(dst),
+                                                               static_cast<const W*>(src), nxm1, nym1, ld);
+        else
+            repack_kernel<W, false><<<(int)blocks, 256, 0, s>>>(static_cast<W*>(dst),
+                                                                static_cast<const W*>(src), nxm1, nym1, ld);
+    };
+    if (esz == 8) go(double());
+    else go(float());
     return cudaGetLastError();
+}
+
+bool on_device(const void* ptr) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, ptr) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice;
 }
 
 // Device buffers and pinned host buffers (read or written in place over the
@@ -469,6 +516,8 @@ cudaError_t copy_out(void* dense, const void* padded, int ld, int nxm1, int nym1
                                             cudaStream_t);                          \
     template cudaError_t launch_prolong<T>(const T*, int, T*, int, int, int, int,   \
                                            cudaStream_t);                            \
+    template cudaError_t launch_restrict_dense<T>(const T*, T*, int, int, int, cudaStream_t); \
+    template cudaError_t launch_prolong_dense<T>(const T*, T*, int, int, int, cudaStream_t); \
     template cudaError_t launch_cfl_max<T>(const T*, int, int, int, int, double,     \
                                            double, unsigned long long*, cudaStream_t); \
     template cudaError_t launch_accumulate<T>(double*, const T*, size_t, cudaStream_t); \
