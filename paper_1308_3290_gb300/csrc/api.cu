@@ -918,10 +918,17 @@ qg_status project(qg_ctx* h, const void* win, cudaStream_t s) {
     return project_to<T>(h, win, h->psi, s);
 }
 
+// The TVDRK3 weight of w^n, 1 - b, from the rounded b: the two add up to one
+// exactly (for b = 2/3 the difference is representable).  Rounded apart, 1/3
+// and 2/3 multiplied an FP32 state by 1 + 3e-8 at every step.
+template <typename T>
+T rk_a(double b) {
+    return T(1) - (T)b;
+}
+
 // TVDRK3 stage s: w_out = a w^n + b (w_in + dt G(w_in)).
 template <typename T>
 qg_status stage(qg_ctx* h, int s_idx, cudaStream_t s) {
-    static const double A[3] = {0.0, 0.75, 1.0 / 3.0};
     static const double B[3] = {1.0, 0.25, 2.0 / 3.0};
     void* win = h->w[s_idx];
     void* wout = h->w[(s_idx + 1) % 3];
@@ -944,7 +951,7 @@ qg_status stage(qg_ctx* h, int s_idx, cudaStream_t s) {
         p.c_lapx = (T)(1.0 / (h->Re * h->dx * h->dx));
         p.c_lapy = (T)(1.0 / (h->Re * h->dy * h->dy));
         p.dt = (T)h->dt;
-        p.a = (T)A[s_idx];
+        p.a = rk_a<T>(B[s_idx]);
         p.b = (T)B[s_idx];
         QG_TRY(launch_fine_stage<T>(static_cast<const T*>(h->psi),
                                     static_cast<const T*>(win),
@@ -967,7 +974,7 @@ qg_status stage(qg_ctx* h, int s_idx, cudaStream_t s) {
         p.A_dy2 = (T)(A2 / (h->dy * h->dy));
         p.sigma = (T)h->sigma;
         p.dt = (T)h->dt;
-        p.a = (T)A[s_idx];
+        p.a = rk_a<T>(B[s_idx]);
         p.b = (T)B[s_idx];
         const size_t P = h->plane_f;
         QG_TRY(launch_fine_stage2<T>(plane<T>(h->psi, P, 0), plane<T>(h->psi, P, 1),
@@ -986,7 +993,6 @@ qg_status stage(qg_ctx* h, int s_idx, cudaStream_t s) {
 // leaves R^l Q_i^(s+1) in that layer's partial planes.
 template <typename T>
 qg_status stage_fused2(qg_ctx* h, int s_idx, const LevelTables& t, cudaStream_t s) {
-    static const double A[3] = {0.0, 0.75, 1.0 / 3.0};
     static const double B[3] = {1.0, 0.25, 2.0 / 3.0};
     void* win = h->w[s_idx];
     void* wout = h->w[(s_idx + 1) % 3];
@@ -1021,7 +1027,7 @@ qg_status stage_fused2(qg_ctx* h, int s_idx, const LevelTables& t, cudaStream_t 
         p.c_lapx = (T)(Av / (h->dx * h->dx));
         p.c_lapy = (T)(Av / (h->dy * h->dy));
         p.dt = (T)h->dt;
-        p.a = (T)A[s_idx];
+        p.a = rk_a<T>(B[s_idx]);
         p.b = (T)B[s_idx];
         p.inv_Ro = (T)(1.0 / h->Ro);
         p.k_p = (T)((L == 0 ? h->Fr / h->delta : h->Fr / (1.0 - h->delta)) / h->Ro);
@@ -1053,7 +1059,6 @@ qg_status stage_fused2(qg_ctx* h, int s_idx, const LevelTables& t, cudaStream_t 
 // partial planes for the next stage.
 template <typename T>
 qg_status stage_fused(qg_ctx* h, int s_idx, cudaStream_t s) {
-    static const double A[3] = {0.0, 0.75, 1.0 / 3.0};
     static const double B[3] = {1.0, 0.25, 2.0 / 3.0};
     void* win = h->w[s_idx];
     void* wout = h->w[(s_idx + 1) % 3];
@@ -1096,7 +1101,7 @@ qg_status stage_fused(qg_ctx* h, int s_idx, cudaStream_t s) {
     p.c_lapx = (T)(1.0 / (h->Re * h->dx * h->dx));
     p.c_lapy = (T)(1.0 / (h->Re * h->dy * h->dy));
     p.dt = (T)h->dt;
-    p.a = (T)A[s_idx];
+    p.a = rk_a<T>(B[s_idx]);
     p.b = (T)B[s_idx];
     p.psi_o = nullptr;
     p.inv_Ro = p.k_p = p.drag = T(0);
@@ -1894,20 +1899,60 @@ qg_status qg_step_kernel_count(qg_handle h, int64_t* count) {
     return QG_OK;
 }
 
+// The sums of launch_diagnostics over w^n and h->psi (+ lo), into h->dout.
+static qg_status diagnostics_sums(qg_ctx* h, const float* lo) {
+    QG_TRY(h->dtype == QG_F64
+               ? launch_diagnostics<double>((const double*)h->psi, nullptr, (const double*)h->w[0],
+                                            h->nx, h->ny, h->ldf, h->dpart, diag_blocks(), h->dout,
+                                            h->stream)
+               : launch_diagnostics<float>((const float*)h->psi, lo, (const float*)h->w[0], h->nx,
+                                           h->ny, h->ldf, h->dpart, diag_blocks(), h->dout,
+                                           h->stream));
+    return QG_OK;
+}
+
+// After project: h->psi + *lo is the streamfunction of w^n refined once on
+// the elliptic grid (FP32, one layer, sine transforms).  *scratch holds lo;
+// the caller frees it.
+static qg_status refine_psi(qg_ctx* h, void** scratch, const float** lo) {
+    const LevelTables* t = nullptr;
+    qg_status st = get_level(h, h->levels, &t);
+    if (st != QG_OK) return fail(h, st);
+    const size_t pc = h->plane_c;
+    QG_TRY(scratch_alloc(h, scratch, (2 * pc + h->plane_f) * sizeof(float)));
+    float *r = static_cast<float*>(*scratch), *d = r + pc, *l = d + pc;
+    float* psi = static_cast<float*>(h->levels ? h->cpsi : h->psi);
+    cudaError_t e = cudaMemsetAsync(d, 0, pc * sizeof(float), h->stream);
+    if (e == cudaSuccess)
+        e = launch_residual(static_cast<const float*>(h->w[0]), h->ldf, psi, r, t->ldc, t->mx, t->my,
+                            h->levels, 1.0 / (t->dxc * t->dxc), 1.0 / (t->dyc * t->dyc), h->stream);
+    if (e == cudaSuccess)
+        st = solve_level<float>(h, *t, r, h->ct, h->ld_t, h->plane_t, h->cw, d, pc, h->stream);
+    if (e == cudaSuccess && st == QG_OK)
+        e = launch_prolong_pair(psi, d, t->ldc, static_cast<float*>(h->psi), l, h->ldf, h->nx, h->ny,
+                                h->levels, h->stream);
+    if (e != cudaSuccess || st != QG_OK) cudaFreeAsync(*scratch, h->stream);
+    if (st != QG_OK) return st;
+    QG_TRY(e);
+    *lo = l;
+    return QG_OK;
+}
+
 qg_status qg_diagnostics(qg_handle h, double* ke, double* enstrophy, double* max_vel) {
     NvtxRange nvtx_range("qg_diagnostics");
     if (!h) return QG_ERR_ARG;
     if (h->latched != QG_OK) return qg_last_error(h);
     qg_status s = project_any(h, h->w[0], h->stream);
     if (s != QG_OK) return s;
-    if (h->dtype == QG_F64)
-        QG_TRY(launch_diagnostics<double>((const double*)h->psi, (const double*)h->w[0], h->nx,
-                                          h->ny, h->ldf, h->dx, h->dy, h->dpart, diag_blocks(),
-                                          h->dout, h->stream));
-    else
-        QG_TRY(launch_diagnostics<float>((const float*)h->psi, (const float*)h->w[0], h->nx,
-                                         h->ny, h->ldf, h->dx, h->dy, h->dpart, diag_blocks(),
-                                         h->dout, h->stream));
+    void* scratch = nullptr;
+    const float* lo = nullptr;
+    if (h->dtype == QG_F32 && h->layers == 1 && h->solver == QG_SOLVER_FFT) {
+        s = refine_psi(h, &scratch, &lo);
+        if (s != QG_OK) return s;
+    }
+    s = diagnostics_sums(h, lo);
+    if (scratch) cudaFreeAsync(scratch, h->stream);
+    if (s != QG_OK) return s;
     QG_TRY(cudaMemcpyAsync(h->hout, h->dout, sizeof(double) * 5, cudaMemcpyDeviceToHost, h->stream));
     QG_TRY(cudaStreamSynchronize(h->stream));
     {
@@ -1932,14 +1977,8 @@ qg_status qg_energy_accumulate(qg_handle h, double scale, double* acc) {
     if (h->latched != QG_OK) return qg_last_error(h);
     qg_status s = project_any(h, h->w[0], h->stream);
     if (s != QG_OK) return s;
-    if (h->dtype == QG_F64)
-        QG_TRY(launch_diagnostics<double>((const double*)h->psi, (const double*)h->w[0], h->nx,
-                                          h->ny, h->ldf, h->dx, h->dy, h->dpart, diag_blocks(),
-                                          h->dout, h->stream));
-    else
-        QG_TRY(launch_diagnostics<float>((const float*)h->psi, (const float*)h->w[0], h->nx,
-                                         h->ny, h->ldf, h->dx, h->dy, h->dpart, diag_blocks(),
-                                         h->dout, h->stream));
+    s = diagnostics_sums(h, nullptr);
+    if (s != QG_OK) return s;
     // E = 1/2 dx dy (sx/dx^2 + sy/dy^2), as qg_diagnostics forms it
     const double c0 = scale * 0.5 * h->dy / h->dx, c1 = scale * 0.5 * h->dx / h->dy;
     QG_TRY(launch_energy_add(h->dout, c0, c1, acc, h->stream));
@@ -2042,8 +2081,8 @@ qg_status adjoint_one(qg_ctx* h, const void* w) {
     const T* wn = static_cast<const T*>(w);
     const T* frow = static_cast<const T*>(h->frow);
     const T* f2d = static_cast<const T*>(h->f2d);
-    static const double RA[3] = {0.0, 0.75, 1.0 / 3.0};
     static const double RB[3] = {1.0, 0.25, 2.0 / 3.0};
+    const double RA[3] = {rk_a<T>(RB[0]), rk_a<T>(RB[1]), rk_a<T>(RB[2])};
     // forward stages
     qg_status st = project_to<T>(h, wn, B[Tape::P0], s);
     if (st != QG_OK) return st;
@@ -2333,7 +2372,6 @@ std::vector<int> batch_engines(qg_ensemble e, const EnsSolveGroup& g) {
 
 template <typename T>
 FusedParams<T> fused_params(qg_ctx* h, int s_idx, const LevelTables& t) {
-    static const double A[3] = {0.0, 0.75, 1.0 / 3.0};
     static const double B[3] = {1.0, 0.25, 2.0 / 3.0};
     FusedParams<T> p = {};
     p.nx = h->nx;
@@ -2354,7 +2392,7 @@ FusedParams<T> fused_params(qg_ctx* h, int s_idx, const LevelTables& t) {
     p.c_lapx = (T)(1.0 / (h->Re * h->dx * h->dx));
     p.c_lapy = (T)(1.0 / (h->Re * h->dy * h->dy));
     p.dt = (T)h->dt;
-    p.a = (T)A[s_idx];
+    p.a = rk_a<T>(B[s_idx]);
     p.b = (T)B[s_idx];
     p.psi_o = nullptr;
     p.inv_Ro = p.k_p = p.drag = T(0);

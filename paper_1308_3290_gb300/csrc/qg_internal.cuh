@@ -334,9 +334,14 @@ cudaError_t launch_fine_stage2(const T* psi1, const T* psi2, const T* q1,
 // differences of psi along x and y, of w^2, and per-CTA maxima of |psi_x|,
 // |psi_y|; then one CTA folds them in a fixed order into out[0..3].
 template <typename T>
-cudaError_t launch_diagnostics(const T* psi, const T* w, int nx, int ny, int ld,
-                               double dx, double dy, double* partial,
-                               int nblocks, double* out, cudaStream_t s);
+cudaError_t launch_diagnostics(const T* psi, const T* lo, const T* w, int nx, int ny, int ld,
+                               double* partial, int nblocks, double* out, cudaStream_t s);
+// One step of iterative refinement of an FP32 psi (diag.cu): r = R^l w -
+// lap_h psi, and the prolonged sum of psi and its correction as hi + lo.
+cudaError_t launch_residual(const float* w, int ldf, const float* psi, float* r, int ld, int mx,
+                            int my, int levels, double cx, double cy, cudaStream_t s);
+cudaError_t launch_prolong_pair(const float* c, const float* d, int ldc, float* hi, float* lo,
+                                int ldf, int nx, int ny, int levels, cudaStream_t s);
 int diag_blocks();
 // acc[0] += c0 out[0] + c1 out[1] (out: the FP64 results of launch_diagnostics)
 cudaError_t launch_energy_add(const double* out, double c0, double c1, double* acc,
