@@ -53,10 +53,12 @@ class MeanKineticEnergy(torch.autograd.Function):
         lam = torch.zeros(ctx.shape, dtype=ctx.dtype, device=ctx.device)
         gF = torch.zeros_like(lam)
         K = N - n0 + 1
-        for n in range(N, 0, -1):
-            if n >= n0:
-                qg.qg_energy_gradient(h, 1.0 / K, lam)
+        # dE/dw joins at n = N..n0; the steps below n0 go back in one call
+        for n in range(N, max(n0, 1) - 1, -1):
+            qg.qg_energy_gradient(h, 1.0 / K, lam)
             qg.qg_adjoint_step(h, 1, lam, gF)
+        if n0 > 1:
+            qg.qg_adjoint_step(h, n0 - 1, lam, gF)
         qg.qg_synchronize(h)
         qg.qg_tape_end(h)
         return grad_J.to(gF.dtype) * gF, None, None, None, None, None

@@ -73,7 +73,7 @@ struct MGPlan {
 
 // Forward states kept for the adjoint (one layer): the state at every
 // `every`-th step, the states of the segment being reversed (every > 1), the
-// handle's state when the reversal began, and the adjoint's work fields.
+// handle's state when the reversal began.
 struct Tape {
     int64_t every = 1, max_steps = 0, recorded = 0, cursor = 0;
     bool reversing = false;
@@ -81,9 +81,26 @@ struct Tape {
     std::vector<void*> seg;
     int64_t seg_start = -1;
     void* live = nullptr;
-    enum { W1, W2, P0, P1, P2, U, PHI, L0, L1, ACC, GF, NBUF };
+    void* block = nullptr;         // the memory of the states
+    bool pooled = false;           // block came from the handle's pool
+};
+
+// The adjoint's work fields, kept with the handle from the first tape on (the
+// captured graphs refer to them): states and streamfunctions of a step's
+// stages, the solve's result, lambda of the three stages, the forcing
+// gradient, partial planes.
+struct AdjWork {
+    enum { W0, W1, W2, P0, P1, P2, PHI, U, L0, L1, L2, GF, NBUF };
     void* buf[NBUF] = {};
-    std::vector<void*> allocs;
+    void* part = nullptr;          // 4 planes (l >= 1)
+};
+
+// A sequence of launches on the handle's own buffers, captured at its second
+// use since the handle's graphs were last dropped (a single use is cheaper
+// launched as it is).
+struct Replay {
+    cudaGraphExec_t exec = nullptr;
+    int uses = 0;
 };
 
 struct qg_ctx {
@@ -155,6 +172,8 @@ struct qg_ctx {
     int* derr = nullptr;           // device error flag of bounded waits
     unsigned* dbar = nullptr;      // grid-barrier counters of the solve kernel
     Tape* tape = nullptr;          // adjoint tape (qg_tape_begin .. qg_tape_end)
+    AdjWork adj;
+    Replay adj_step, adj_energy, energy_sums;
     double cfl = 0.0;              // > 0: adaptive step (Eq. dt) with this CFL number
     double time_host = 0.0;        // model time of two-layer handles (fixed dt)
     bool stats = false;            // accumulate the first-stage psi of every step
@@ -533,7 +552,7 @@ qg_status mg_solve_level(qg_ctx* h, const LevelTables& t, const void* in, int np
 template <typename T>
 qg_status solve_level(qg_ctx* h, const LevelTables& t, const void* in, void* tr, int ld_tr,
                       size_t pl_tr, void* work, void* out, size_t pl, cudaStream_t s,
-                      int nparts = 1, int engine = 0) {
+                      int nparts = 1, int tile_ry = 0, int tile_rows = 0) {
     using C = typename Cx<T>::type;
     if (h->solver == QG_SOLVER_MULTIGRID && h->layers == 1)
         return mg_solve_level<T>(h, t, in, nparts, out, pl, s, false);
@@ -551,14 +570,24 @@ qg_status solve_level(qg_ctx* h, const LevelTables& t, const void* in, void* tr,
     P.nin = nparts;
     P.part_px = P.part_py = 1;
     if (nparts > 1) {
-        P.part_px = fine_part_period_x(h->levels, h->fine_ry);
-        P.part_py = fine_part_period_y(h->levels, h->fine_rows);
+        // (the tile that wrote the planes: the step's, unless given)
+        P.part_px = fine_part_period_x(h->levels, tile_ry ? tile_ry : h->fine_ry);
+        P.part_py = fine_part_period_y(h->levels, tile_rows ? tile_rows : h->fine_rows);
     }
     P.ld = t.ldc;
     P.ld_tr = ld_tr;
     P.twx = static_cast<const C*>(t.twx);
     P.twy = static_cast<const C*>(t.twy);
-    const int eng = engine ? engine : engine_for(h, t.mx, t.my);
+    int eng = engine_for(h, t.mx, t.my);
+    // the barrier stall needs a solve with a grid barrier
+    if (h->fault == QG_FAULT_BARRIER_STALL && (eng == kDenseEngine || eng == kStreamEngine)) {
+        const int b = engine_rule(t.mx, t.my);
+        for (int c : {b, 20 - b})
+            if (solve_engine_supports(t.mx, t.my, sizeof(T), c)) {
+                eng = c;
+                break;
+            }
+    }
     if (is_warp_engine(eng)) {
         P.ptx = static_cast<const C*>(t.ptx[eng - 32]);
         P.pty = static_cast<const C*>(t.pty[eng - 32]);
@@ -926,7 +955,8 @@ T rk_a(double b) {
     return T(1) - (T)b;
 }
 
-// TVDRK3 stage s: w_out = a w^n + b (w_in + dt G(w_in)).
+// TVDRK3 stage s of a two-layer handle at l = 0 (the other handles' stages are
+// fused): w_out = a w^n + b (w_in + dt G(w_in)).
 template <typename T>
 qg_status stage(qg_ctx* h, int s_idx, cudaStream_t s) {
     static const double B[3] = {1.0, 0.25, 2.0 / 3.0};
@@ -941,48 +971,28 @@ qg_status stage(qg_ctx* h, int s_idx, cudaStream_t s) {
                                     h->plane_f * h->layers, s));
     }
     KTimer kt(h, s, QG_K_FINE);
-    if (h->layers == 1) {
-        StageParams<T> p;
-        p.nx = h->nx;
-        p.ny = h->ny;
-        p.ld = h->ldf;
-        p.c_jac = (T)(1.0 / (12.0 * h->dx * h->dy));
-        p.c_beta = (T)(1.0 / (12.0 * h->Ro * h->dx));
-        p.c_lapx = (T)(1.0 / (h->Re * h->dx * h->dx));
-        p.c_lapy = (T)(1.0 / (h->Re * h->dy * h->dy));
-        p.dt = (T)h->dt;
-        p.a = rk_a<T>(B[s_idx]);
-        p.b = (T)B[s_idx];
-        QG_TRY(launch_fine_stage<T>(static_cast<const T*>(h->psi),
-                                    static_cast<const T*>(win),
-                                    static_cast<const T*>(h->w[0]),
-                                    static_cast<T*>(wout),
-                                    static_cast<const T*>(h->frow),
-                                    static_cast<const T*>(h->f2d), p, s));
-    } else {
-        StageParams2<T> p;
-        p.nx = h->nx;
-        p.ny = h->ny;
-        p.ld = h->ldf;
-        p.c_jac = (T)(1.0 / (12.0 * h->dx * h->dy));
-        p.c_beta = (T)(1.0 / (12.0 * h->dx));
-        p.inv_Ro = (T)(1.0 / h->Ro);
-        p.f1 = (T)(h->Fr / h->delta);
-        p.f2 = (T)(h->Fr / (1.0 - h->delta));
-        const double A2 = h->Ro / h->Re;
-        p.A_dx2 = (T)(A2 / (h->dx * h->dx));
-        p.A_dy2 = (T)(A2 / (h->dy * h->dy));
-        p.sigma = (T)h->sigma;
-        p.dt = (T)h->dt;
-        p.a = rk_a<T>(B[s_idx]);
-        p.b = (T)B[s_idx];
-        const size_t P = h->plane_f;
-        QG_TRY(launch_fine_stage2<T>(plane<T>(h->psi, P, 0), plane<T>(h->psi, P, 1),
-                                     plane<T>(win, P, 0), plane<T>(win, P, 1),
-                                     plane<T>(h->w[0], P, 0), plane<T>(h->w[0], P, 1),
-                                     plane<T>(wout, P, 0), plane<T>(wout, P, 1),
-                                     static_cast<const T*>(h->frow), p, s));
-    }
+    StageParams2<T> p;
+    p.nx = h->nx;
+    p.ny = h->ny;
+    p.ld = h->ldf;
+    p.c_jac = (T)(1.0 / (12.0 * h->dx * h->dy));
+    p.c_beta = (T)(1.0 / (12.0 * h->dx));
+    p.inv_Ro = (T)(1.0 / h->Ro);
+    p.f1 = (T)(h->Fr / h->delta);
+    p.f2 = (T)(h->Fr / (1.0 - h->delta));
+    const double A2 = h->Ro / h->Re;
+    p.A_dx2 = (T)(A2 / (h->dx * h->dx));
+    p.A_dy2 = (T)(A2 / (h->dy * h->dy));
+    p.sigma = (T)h->sigma;
+    p.dt = (T)h->dt;
+    p.a = rk_a<T>(B[s_idx]);
+    p.b = (T)B[s_idx];
+    const size_t P = h->plane_f;
+    QG_TRY(launch_fine_stage2<T>(plane<T>(h->psi, P, 0), plane<T>(h->psi, P, 1),
+                                 plane<T>(win, P, 0), plane<T>(win, P, 1),
+                                 plane<T>(h->w[0], P, 0), plane<T>(h->w[0], P, 1),
+                                 plane<T>(wout, P, 0), plane<T>(wout, P, 1),
+                                 static_cast<const T*>(h->frow), p, s));
     return QG_OK;
 }
 
@@ -1166,6 +1176,10 @@ qg_status project_any(qg_ctx* h, const void* win, cudaStream_t s) {
 }
 
 void drop_graph(qg_ctx* h) {
+    for (Replay* r : {&h->adj_step, &h->adj_energy, &h->energy_sums}) {
+        if (r->exec) cudaGraphExecDestroy(r->exec);
+        *r = Replay();
+    }
     ++h->graph_gen;
     if (h->gexec) cudaGraphExecDestroy(h->gexec);
     if (h->graph) cudaGraphDestroy(h->graph);
@@ -1191,6 +1205,29 @@ qg_status build_graph(qg_ctx* h) {
     if (e != cudaSuccess) return cuda_status(h, e);
     h->graph = g;
     QG_TRY(cudaGraphInstantiate(&h->gexec, g, 0));
+    return QG_OK;
+}
+
+// Run `body` (a qg_status of the stream it enqueues on) on the handle's
+// stream: as it is the first time, from a captured graph after that.
+template <typename F>
+qg_status replay(qg_ctx* h, Replay& r, F body) {
+    if (!r.exec && ++r.uses > 1) {
+        QG_TRY(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
+        const qg_status st = body(h->cap);
+        cudaGraph_t g = nullptr;
+        const cudaError_t e = cudaStreamEndCapture(h->cap, &g);
+        if (st != QG_OK) {
+            if (g) cudaGraphDestroy(g);
+            return st;
+        }
+        if (e != cudaSuccess) return cuda_status(h, e);
+        const cudaError_t ei = cudaGraphInstantiate(&r.exec, g, 0);
+        cudaGraphDestroy(g);
+        QG_TRY(ei);
+    }
+    if (!r.exec) return body(h->stream);
+    QG_TRY(cudaGraphLaunch(r.exec, h->stream));
     return QG_OK;
 }
 
@@ -1488,7 +1525,8 @@ qg_status qg_set_forcing(qg_handle h, const void* forcing) {
     if (!h) return QG_ERR_ARG;
     if (h->layers != 1) return QG_ERR_UNSUPPORTED;
     if (h->latched != QG_OK) return qg_last_error(h);
-    drop_graph(h);
+    // the captured step holds the field's address, not its values
+    if ((forcing != nullptr) != (h->f2d != nullptr)) drop_graph(h);
     if (!forcing) {
         h->f2d = nullptr;   // f2d_buf stays allocated for reuse
         return QG_OK;
@@ -1900,14 +1938,14 @@ qg_status qg_step_kernel_count(qg_handle h, int64_t* count) {
 }
 
 // The sums of launch_diagnostics over w^n and h->psi (+ lo), into h->dout.
-static qg_status diagnostics_sums(qg_ctx* h, const float* lo) {
+static qg_status diagnostics_sums(qg_ctx* h, const float* lo, cudaStream_t s) {
     QG_TRY(h->dtype == QG_F64
                ? launch_diagnostics<double>((const double*)h->psi, nullptr, (const double*)h->w[0],
                                             h->nx, h->ny, h->ldf, h->dpart, diag_blocks(), h->dout,
-                                            h->stream)
+                                            s)
                : launch_diagnostics<float>((const float*)h->psi, lo, (const float*)h->w[0], h->nx,
                                            h->ny, h->ldf, h->dpart, diag_blocks(), h->dout,
-                                           h->stream));
+                                           s));
     return QG_OK;
 }
 
@@ -1950,7 +1988,7 @@ qg_status qg_diagnostics(qg_handle h, double* ke, double* enstrophy, double* max
         s = refine_psi(h, &scratch, &lo);
         if (s != QG_OK) return s;
     }
-    s = diagnostics_sums(h, lo);
+    s = diagnostics_sums(h, lo, h->stream);
     if (scratch) cudaFreeAsync(scratch, h->stream);
     if (s != QG_OK) return s;
     QG_TRY(cudaMemcpyAsync(h->hout, h->dout, sizeof(double) * 5, cudaMemcpyDeviceToHost, h->stream));
@@ -1975,9 +2013,10 @@ qg_status qg_energy_accumulate(qg_handle h, double scale, double* acc) {
     NvtxRange nvtx_range("qg_energy_accumulate");
     if (!h || !acc || !std::isfinite(scale)) return QG_ERR_ARG;
     if (h->latched != QG_OK) return qg_last_error(h);
-    qg_status s = project_any(h, h->w[0], h->stream);
-    if (s != QG_OK) return s;
-    s = diagnostics_sums(h, nullptr);
+    qg_status s = replay(h, h->energy_sums, [&](cudaStream_t q) {
+        const qg_status e = project_any(h, h->w[0], q);
+        return e != QG_OK ? e : diagnostics_sums(h, nullptr, q);
+    });
     if (s != QG_OK) return s;
     // E = 1/2 dx dy (sx/dx^2 + sy/dy^2), as qg_diagnostics forms it
     const double c0 = scale * 0.5 * h->dy / h->dx, c1 = scale * 0.5 * h->dx / h->dy;
@@ -1991,29 +2030,8 @@ qg_status qg_energy_accumulate(qg_handle h, double scale, double* acc) {
 
 namespace {
 
-void tape_free_all(Tape* tp) {
-    for (void* p : tp->allocs) cudaFree(p);
-    delete tp;
-}
-
 template <typename T>
-StageParams<T> stage_params(const qg_ctx* h, double a, double b) {
-    StageParams<T> p;
-    p.nx = h->nx;
-    p.ny = h->ny;
-    p.ld = h->ldf;
-    p.c_jac = (T)(1.0 / (12.0 * h->dx * h->dy));
-    p.c_beta = (T)(1.0 / (12.0 * h->Ro * h->dx));
-    p.c_lapx = (T)(1.0 / (h->Re * h->dx * h->dx));
-    p.c_lapy = (T)(1.0 / (h->Re * h->dy * h->dy));
-    p.dt = (T)h->dt;
-    p.a = (T)a;
-    p.b = (T)b;
-    return p;
-}
-
-template <typename T>
-AdjParams<T> adj_params(const qg_ctx* h, double a, double b) {
+AdjParams<T> adj_params(const qg_ctx* h, double b) {
     AdjParams<T> p;
     p.nx = h->nx;
     p.ny = h->ny;
@@ -2023,7 +2041,6 @@ AdjParams<T> adj_params(const qg_ctx* h, double a, double b) {
     p.c_lapx = (T)(1.0 / (h->Re * h->dx * h->dx));
     p.c_lapy = (T)(1.0 / (h->Re * h->dy * h->dy));
     p.dt = (T)h->dt;
-    p.a = (T)a;
     p.b = (T)b;
     p.inv_dx2 = (T)(1.0 / (h->dx * h->dx));
     p.inv_dy2 = (T)(1.0 / (h->dy * h->dy));
@@ -2043,8 +2060,7 @@ qg_status tape_state(qg_ctx* h, int64_t t, const void** out) {
     const int64_t start = t / tp->every * tp->every;
     if (tp->seg_start != start) {
         if (!tp->live) {
-            QG_TRY(cudaMalloc(&tp->live, bytes + 4 * sizeof(double)));
-            tp->allocs.push_back(tp->live);
+            tp->live = static_cast<char*>(tp->block) + (tp->ckpt.size() + tp->seg.size()) * bytes;
             QG_TRY(cudaMemcpyAsync(tp->live, h->w[0], bytes, cudaMemcpyDeviceToDevice, h->stream));
             QG_TRY(cudaMemcpyAsync(static_cast<char*>(tp->live) + bytes, h->dclock,
                                    4 * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
@@ -2070,44 +2086,87 @@ qg_status tape_state(qg_ctx* h, int64_t t, const void** out) {
     return QG_OK;
 }
 
-// lam(t) -> lam(t - 1) through the step from w^n = w (tape time t - 1): the
-// three stages are recomputed (w^(1), w^(2), psi^(0..2)), then reversed.
 template <typename T>
-qg_status adjoint_one(qg_ctx* h, const void* w) {
-    Tape* tp = h->tape;
-    cudaStream_t s = h->stream;
-    T* B[Tape::NBUF];
-    for (int k = 0; k < Tape::NBUF; ++k) B[k] = static_cast<T*>(tp->buf[k]);
-    const T* wn = static_cast<const T*>(w);
-    const T* frow = static_cast<const T*>(h->frow);
-    const T* f2d = static_cast<const T*>(h->f2d);
+FusedParams<T> fused_params(qg_ctx* h, int s_idx, const LevelTables& t);
+
+// A w: the solve of `nparts` partial planes (or of a field) into `out`, a
+// field of the elliptic grid (l = 0: the fine grid).
+template <typename T>
+qg_status adj_solve(qg_ctx* h, const LevelTables& t, const void* in, int nparts, void* out,
+                    cudaStream_t s) {
+    return solve_level<T>(h, t, in, h->ct, h->ld_t, h->plane_t, h->cw, out,
+                          h->levels ? h->plane_c : h->plane_f, s, nparts, 1,
+                          node_tile_rows(h->levels));
+}
+
+// The streamfunction on the elliptic grid of the fine state w: into `out`.
+template <typename T>
+qg_status adj_project(qg_ctx* h, const LevelTables& t, const void* w, void* out, cudaStream_t s) {
+    if (h->levels == 0) return adj_solve<T>(h, t, w, 1, out, s);
+    QG_TRY(launch_restrict<T>(static_cast<const T*>(w), h->ldf, static_cast<T*>(h->adj.part), t.ldc,
+                              t.mx, t.my, h->levels, s));
+    return adj_solve<T>(h, t, h->adj.part, 1, out, s);
+}
+
+template <typename T>
+AdjOut<T> adj_out(qg_ctx* h, const LevelTables& t) {
+    AdjOut<T> o = {};
+    for (int q = 0; q < 4; ++q)
+        o.part[q] = h->adj.part ? plane<T>(h->adj.part, h->plane_c, q) : nullptr;
+    o.ldc = t.ldc;
+    o.fine = static_cast<T*>(h->adj.buf[AdjWork::U]);
+    return o;
+}
+
+// lam(t) -> lam(t - 1) through the step from w^n = W0 (tape time t - 1), in
+// place in L0: the stages are recomputed (W1, W2, P0..P2 on the elliptic
+// grid), then reversed.  Every state update runs with one node per thread.
+template <typename T>
+qg_status adjoint_one(qg_ctx* h, cudaStream_t s) {
+    T* B[AdjWork::NBUF];
+    for (int k = 0; k < AdjWork::NBUF; ++k) B[k] = static_cast<T*>(h->adj.buf[k]);
+    const LevelTables* t = nullptr;
+    qg_status st = get_level(h, h->levels, &t);
+    if (st != QG_OK) return fail(h, st);
+    const AdjOut<T> src = adj_out<T>(h, *t);
+    const void* rhs = h->levels ? h->adj.part : h->adj.buf[AdjWork::U];
+    const int nparts = h->levels ? 4 : 1;
     static const double RB[3] = {1.0, 0.25, 2.0 / 3.0};
-    const double RA[3] = {rk_a<T>(RB[0]), rk_a<T>(RB[1]), rk_a<T>(RB[2])};
-    // forward stages
-    qg_status st = project_to<T>(h, wn, B[Tape::P0], s);
-    if (st != QG_OK) return st;
-    QG_TRY(launch_fine_stage<T>(B[Tape::P0], wn, wn, B[Tape::W1], frow, f2d,
-                                stage_params<T>(h, RA[0], RB[0]), s));
-    if ((st = project_to<T>(h, B[Tape::W1], B[Tape::P1], s)) != QG_OK) return st;
-    QG_TRY(launch_fine_stage<T>(B[Tape::P1], B[Tape::W1], wn, B[Tape::W2], frow, f2d,
-                                stage_params<T>(h, RA[1], RB[1]), s));
-    if ((st = project_to<T>(h, B[Tape::W2], B[Tape::P2], s)) != QG_OK) return st;
-    // reverse: lam in L0, result in ACC
-    QG_TRY(cudaMemsetAsync(B[Tape::ACC], 0, h->plane_f * h->esz, s));
-    const T* ws[3] = {wn, B[Tape::W1], B[Tape::W2]};
-    const T* ps[3] = {B[Tape::P0], B[Tape::P1], B[Tape::P2]};
-    T* lam = B[Tape::L0];
-    T* nxt = B[Tape::L1];
-    for (int k = 2; k >= 0; --k) {
-        const AdjParams<T> p = adj_params<T>(h, RA[k], RB[k]);
-        QG_TRY(launch_adj_source<T>(ws[k], lam, B[Tape::U], p, s));
-        if ((st = project_to<T>(h, B[Tape::U], B[Tape::PHI], s)) != QG_OK) return st;
-        T* out = k == 0 ? B[Tape::ACC] : nxt;
-        QG_TRY(launch_adj_stage<T>(ps[k], lam, B[Tape::PHI], out, B[Tape::ACC], B[Tape::GF], p,
-                                   k == 0, s));
-        if (k > 0) std::swap(lam, nxt);
+    T* const W[3] = {B[AdjWork::W0], B[AdjWork::W1], B[AdjWork::W2]};
+    T* const P[3] = {B[AdjWork::P0], B[AdjWork::P1], B[AdjWork::P2]};
+    if ((st = adj_project<T>(h, *t, W[0], P[0], s)) != QG_OK) return st;
+    for (int k = 0; k < 2; ++k) {
+        FusedParams<T> p = fused_params<T>(h, k, *t);
+        p.psi = P[k];
+        p.w = W[k];
+        p.wn = W[0];
+        p.wout = W[k + 1];
+        for (int q = 0; q < 4; ++q) p.part[q] = src.part[q];
+        p.umax = nullptr;
+        p.last_stage = 0;
+        QG_TRY(launch_fine_node<T>(p, h->levels, s));
+        st = adj_solve<T>(h, *t, h->levels ? h->adj.part : W[k + 1], nparts, P[k + 1], s);
+        if (st != QG_OK) return st;
     }
-    std::swap(tp->buf[Tape::L0], tp->buf[Tape::ACC]);
+    const T* lam[3] = {B[AdjWork::L2], B[AdjWork::L1], B[AdjWork::L0]};
+    T* const next[3] = {B[AdjWork::L0], B[AdjWork::L2], B[AdjWork::L1]};
+    const int ldp = h->levels ? t->ldc : h->ldf;
+    for (int k = 2; k >= 0; --k) {
+        const AdjParams<T> p = adj_params<T>(h, RB[k]);
+        QG_TRY(launch_adj_source<T>(W[k], lam[k], src, p, h->levels, s));
+        if ((st = adj_solve<T>(h, *t, rhs, nparts, B[AdjWork::PHI], s)) != QG_OK) return st;
+        AdjFirst<T> f = {};
+        if (k == 0) {
+            f.lam2 = lam[2];
+            f.lam1 = lam[1];
+            f.g = B[AdjWork::GF];
+            f.a2 = rk_a<T>(RB[2]);
+            f.a1 = rk_a<T>(RB[1]);
+            f.b2 = (T)RB[2];
+            f.b1 = (T)RB[1];
+        }
+        QG_TRY(launch_adj_stage<T>(P[k], B[AdjWork::PHI], ldp, lam[k], next[k], f, p, h->levels, s));
+    }
     return QG_OK;
 }
 
@@ -2117,44 +2176,65 @@ qg_status adjoint_steps(qg_ctx* h, int64_t n, void* lambda, void* dJdF) {
     cudaStream_t s = h->stream;
     const size_t bytes = h->plane_f * h->esz;
     tp->reversing = true;
-    QG_TRY(copy_in(tp->buf[Tape::L0], h->ldf, lambda, h->nx - 1, h->ny - 1, h->esz, s));
-    QG_TRY(cudaMemsetAsync(tp->buf[Tape::GF], 0, bytes, s));
+    void* const* B = h->adj.buf;
+    QG_TRY(copy_in(B[AdjWork::L0], h->ldf, lambda, h->nx - 1, h->ny - 1, h->esz, s));
+    QG_TRY(cudaMemsetAsync(B[AdjWork::GF], 0, bytes, s));
     for (int64_t k = 0; k < n; ++k) {
         const void* w = nullptr;
         qg_status st = tape_state<T>(h, tp->cursor - 1, &w);
         if (st != QG_OK) return st;
-        if ((st = adjoint_one<T>(h, w)) != QG_OK) return st;
+        QG_TRY(cudaMemcpyAsync(B[AdjWork::W0], w, bytes, cudaMemcpyDeviceToDevice, s));
+        st = replay(h, h->adj_step, [&](cudaStream_t q) { return adjoint_one<T>(h, q); });
+        if (st != QG_OK) return st;
         --tp->cursor;
     }
-    QG_TRY(copy_out(lambda, tp->buf[Tape::L0], h->ldf, h->nx - 1, h->ny - 1, h->esz, s));
-    QG_TRY(launch_add_to_dense<T>(static_cast<T*>(dJdF), static_cast<const T*>(tp->buf[Tape::GF]),
-                                  1.0, h->nx, h->ny, h->ldf, s));
+    QG_TRY(copy_out(lambda, B[AdjWork::L0], h->ldf, h->nx - 1, h->ny - 1, h->esz, s));
+    QG_TRY(launch_add_prolonged<T>(static_cast<T*>(dJdF), static_cast<const T*>(B[AdjWork::GF]),
+                                   h->ldf, 1.0, h->nx, h->ny, 0, s));
     return QG_OK;
 }
 
 template <typename T>
 qg_status energy_gradient(qg_ctx* h, double scale, void* g) {
     Tape* tp = h->tape;
-    cudaStream_t s = h->stream;
     const void* w = nullptr;
     qg_status st = tape_state<T>(h, tp->cursor, &w);
     if (st != QG_OK) return st;
-    T* P = static_cast<T*>(tp->buf[Tape::P0]);
-    T* U = static_cast<T*>(tp->buf[Tape::U]);
-    T* PHI = static_cast<T*>(tp->buf[Tape::PHI]);
-    if ((st = project_to<T>(h, w, P, s)) != QG_OK) return st;
-    QG_TRY(launch_energy_source<T>(P, U, adj_params<T>(h, 0.0, 0.0), s));
-    if ((st = project_to<T>(h, U, PHI, s)) != QG_OK) return st;
-    QG_TRY(launch_add_to_dense<T>(static_cast<T*>(g), PHI, scale, h->nx, h->ny, h->ldf, s));
+    const LevelTables* t = nullptr;
+    if ((st = get_level(h, h->levels, &t)) != QG_OK) return fail(h, st);
+    void* const* B = h->adj.buf;
+    const int ldp = h->levels ? t->ldc : h->ldf;
+    QG_TRY(cudaMemcpyAsync(B[AdjWork::W0], w, h->plane_f * h->esz, cudaMemcpyDeviceToDevice,
+                           h->stream));
+    st = replay(h, h->adj_energy, [&](cudaStream_t q) -> qg_status {
+        qg_status e = adj_project<T>(h, *t, B[AdjWork::W0], B[AdjWork::P0], q);
+        if (e != QG_OK) return e;
+        QG_TRY(launch_energy_source<T>(static_cast<const T*>(B[AdjWork::P0]), ldp, adj_out<T>(h, *t),
+                                       adj_params<T>(h, 0.0), h->levels, q));
+        return adj_solve<T>(h, *t, h->levels ? h->adj.part : B[AdjWork::U], h->levels ? 4 : 1,
+                            B[AdjWork::PHI], q);
+    });
+    if (st != QG_OK) return st;
+    QG_TRY(launch_add_prolonged<T>(static_cast<T*>(g), static_cast<const T*>(B[AdjWork::PHI]), ldp,
+                                   scale, h->nx, h->ny, h->levels, h->stream));
     return QG_OK;
 }
 
 }  // namespace
 
+constexpr size_t kTapePool = (size_t)256 << 20;
+
 static void tape_release(qg_ctx* h) {
     if (!h->tape) return;
-    cudaStreamSynchronize(h->stream);
-    tape_free_all(h->tape);
+    if (h->tape->block) {
+        if (h->tape->pooled) {
+            cudaFreeAsync(h->tape->block, h->stream);
+        } else {
+            cudaStreamSynchronize(h->stream);
+            cudaFree(h->tape->block);
+        }
+    }
+    delete h->tape;
     h->tape = nullptr;
 }
 
@@ -2170,30 +2250,28 @@ qg_status qg_tape_begin(qg_handle h, int64_t every, int64_t max_steps) {
     if (!tp) return QG_ERR_OOM;
     tp->every = every;
     tp->max_steps = max_steps;
+    // the states in one block (they are copied whole, walls included): from
+    // the handle's pool up to kTapePool bytes (kept by the handle for the next
+    // tape), else an allocation of the tape's own
     const size_t bytes = h->plane_f * h->esz;
-    auto alloc = [&](void** p) {
-        if (cudaMalloc(p, bytes) != cudaSuccess) return false;
-        tp->allocs.push_back(*p);
-        return cudaMemsetAsync(*p, 0, bytes, h->stream) == cudaSuccess;
-    };
+    const size_t nck = (size_t)(max_steps / every) + 1, nseg = every > 1 ? (size_t)every + 1 : 0;
+    const size_t total = (nck + nseg + (every > 1 ? 1 : 0)) * bytes + 4 * sizeof(double);
+    tp->pooled = total <= kTapePool;
     bool ok = true;
-    const int64_t nck = max_steps / every + 1;
-    for (int64_t k = 0; k < nck && ok; ++k) {
-        void* p = nullptr;
-        ok = alloc(&p);
-        if (ok) tp->ckpt.push_back(p);
-    }
-    for (int64_t k = 0; every > 1 && k <= every && ok; ++k) {
-        void* p = nullptr;
-        ok = alloc(&p);
-        if (ok) tp->seg.push_back(p);
-    }
-    for (int k = 0; k < Tape::NBUF && ok; ++k) ok = alloc(&tp->buf[k]);
+    for (int k = 0; k < AdjWork::NBUF && ok; ++k)
+        if (!h->adj.buf[k]) ok = dev_alloc(h, &h->adj.buf[k], bytes) == QG_OK;
+    if (ok && h->levels && !h->adj.part)
+        ok = dev_alloc(h, &h->adj.part, 4 * h->plane_c * h->esz) == QG_OK;
+    if (ok)
+        ok = (tp->pooled ? scratch_alloc(h, &tp->block, total) : cudaMalloc(&tp->block, total)) ==
+             cudaSuccess;
+    for (size_t k = 0; k < nck + nseg && ok; ++k)
+        (k < nck ? tp->ckpt : tp->seg).push_back(static_cast<char*>(tp->block) + k * bytes);
     if (ok) ok = cudaMemcpyAsync(tp->ckpt[0], h->w[0], bytes, cudaMemcpyDeviceToDevice,
                                  h->stream) == cudaSuccess;
     if (!ok) {
-        cudaStreamSynchronize(h->stream);
-        tape_free_all(tp);
+        h->tape = tp;
+        tape_release(h);
         (void)cudaGetLastError();
         return QG_ERR_OOM;
     }

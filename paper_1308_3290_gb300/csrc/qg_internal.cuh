@@ -168,27 +168,6 @@ template <typename T>
 cudaError_t launch_prolong_dense(const T* coarse, T* fine, int nx, int ny, int levels,
                                  cudaStream_t s);
 
-// Constants of one fine-grid stage of the one-layer model.
-template <typename T>
-struct StageParams {
-    int nx, ny, ld;
-    T c_jac;      // 1 / (12 dx dy): Arakawa (J1 + J2 + J3) / 3 / (4 dx dy)
-    T c_beta;     // 1 / (12 Ro dx): closed form of (1/Ro) J(psi, y)
-    T c_lapx;     // 1 / (Re dx^2)
-    T c_lapy;     // 1 / (Re dy^2)
-    T dt;
-    T a;          // weight of w^n in the TVDRK3 combination
-    T b;          // weight of (w^(s) + dt G)
-};
-
-// One TVDRK3 stage on the fine grid: w_out = a w_n + b (w + dt G(psi, w)),
-// G = -J(psi, w) - (1/Ro) J(psi, y) + (1/Re) lap w + F.  F is the per-row
-// forcing `frow` (length ny + 1), or the padded field `f2d` when non-null.
-template <typename T>
-cudaError_t launch_fine_stage(const T* psi, const T* w, const T* wn, T* wout,
-                              const T* frow, const T* f2d,
-                              const StageParams<T>& p, cudaStream_t s);
-
 // Adjoint kernels (adjoint.cu) of the one-layer step.
 template <typename T>
 struct AdjParams {
@@ -198,22 +177,41 @@ struct AdjParams {
     T dt, a, b;           // time step and the stage's TVDRK3 weights
     T inv_dx2, inv_dy2, dxdy;
 };
-// out = J(w, lam) - (1/Ro) J(lam, y)
+// Where a source goes: restricted into partial planes of pitch ldc (levels
+// >= 1; periods of the 16-column tiles of fused_node.cu), or a fine field.
 template <typename T>
-cudaError_t launch_adj_source(const T* w, const T* lam, T* out, const AdjParams<T>& p,
-                              cudaStream_t s);
-// next = [next +] b lam + b dt (J(psi, lam) + (1/Re) lap lam - phi);
-// acc += a lam; g += b dt lam
+struct AdjOut {
+    T* part[4];
+    int ldc;
+    T* fine;
+};
+// What the reversed first stage adds: a_2 lam_2 + a_1 lam_1 to the result and
+// dt (b_2 lam_2 + b_1 lam_1 + b lam) to g.  g null: another stage.
 template <typename T>
-cudaError_t launch_adj_stage(const T* psi, const T* lam, const T* phi, T* next, T* acc, T* g,
-                             const AdjParams<T>& p, bool accumulate, cudaStream_t s);
-// out = -dx dy lap psi
+struct AdjFirst {
+    const T* lam2;
+    const T* lam1;
+    T* g;
+    T a2, a1, b2, b1;
+};
+// J(w, lam) - (1/Ro) J(lam, y) -> out
 template <typename T>
-cudaError_t launch_energy_source(const T* psi, T* out, const AdjParams<T>& p, cudaStream_t s);
-// dense (exchange layout) += scale * padded (interior)
+cudaError_t launch_adj_source(const T* w, const T* lam, const AdjOut<T>& out,
+                              const AdjParams<T>& p, int levels, cudaStream_t s);
+// next = b lam + b dt (J(psi, lam) + (1/Re) lap lam - phi) (+ f), psi and phi
+// on the elliptic grid (pitch ldp); next may be f.lam2
 template <typename T>
-cudaError_t launch_add_to_dense(T* dense, const T* padded, double scale, int nx, int ny, int ld,
-                                cudaStream_t s);
+cudaError_t launch_adj_stage(const T* psi, const T* phi, int ldp, const T* lam, T* next,
+                             const AdjFirst<T>& f, const AdjParams<T>& p, int levels,
+                             cudaStream_t s);
+// -dx dy lap (psi prolonged) -> out
+template <typename T>
+cudaError_t launch_energy_source(const T* psi, int ldp, const AdjOut<T>& out,
+                                 const AdjParams<T>& p, int levels, cudaStream_t s);
+// dense (exchange layout) += scale * (c prolonged `levels` times)
+template <typename T>
+cudaError_t launch_add_prolonged(T* dense, const T* c, int ldc, double scale, int nx, int ny,
+                                 int levels, cudaStream_t s);
 
 // Fused one-layer stage (fused.cu): prolongation of psi on load, the stage
 // update, and restriction of the result into four partial-sum planes.

@@ -1,11 +1,6 @@
-// Fine-grid stage and mapping operators.
-//
-// fine_stage: one TVDRK3 stage (Section 4.2, Eq. TVDRK) of the one-layer
-// vorticity equation on the fine grid, with the Arakawa Jacobian
-// (Section 4.1, Eqs. ja1, j1-j3), the beta term J(psi, y)/Ro, the 5-point
-// dissipation (1/Re) lap w and the wind forcing (Section 2.1, Eq. ge divided
-// by Ro).  restrict / prolong: the mapping operators of Section 3.1 (Eqs. res
-// and pro), l levels at once.
+// The two-layer stage at l = 0, the mapping operators of Section 3.1 (Eqs. res
+// and pro, l levels at once), time means, the velocity maximum of Eq. dt and
+// the copies between the exchange layout and the padded one.
 #include <cuda_runtime.h>
 
 #include "arakawa.cuh"
@@ -14,36 +9,6 @@
 
 namespace qg {
 namespace {
-
-template <typename T>
-__global__ void fine_stage_kernel(const T* __restrict__ psi,
-                                  const T* __restrict__ w, const T* wn,
-                                  T* wout, const T* __restrict__ frow,
-                                  const T* __restrict__ f2d, StageParams<T> p) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x + 1;
-    const int j = blockIdx.y * blockDim.y + threadIdx.y + 1;
-    if (i >= p.nx || j >= p.ny) return;
-    const int ld = p.ld;
-    const size_t c = (size_t)j * ld + i;
-    const T* P = psi + c;
-    const T* Q = w + c;
-    const T pm0 = P[-1], p10 = P[1], p0m = P[-ld], p01 = P[ld];
-    const T pmm = P[-ld - 1], p1m = P[-ld + 1], pm1 = P[ld - 1], p11 = P[ld + 1];
-    const T q00 = Q[0];
-    const T qm0 = Q[-1], q10 = Q[1], q0m = Q[-ld], q01 = Q[ld];
-    const T qmm = Q[-ld - 1], q1m = Q[-ld + 1], qm1 = Q[ld - 1], q11 = Q[ld + 1];
-    const T jac = arakawa_sum(pm0, p10, p0m, p01, pmm, p1m, pm1, p11, qm0, q10,
-                              q0m, q01, qmm, q1m, qm1, q11) * p.c_jac;
-    // (1/Ro) J(psi, y) = (4 c_j + c_{j+1} + c_{j-1}) / (6 Ro),
-    // c = (psi_{i+1} - psi_{i-1}) / (2 dx): Arakawa's form with q = y.
-    const T beta = (T(4) * (p10 - pm0) + (p11 - pm1) + (p1m - pmm)) * p.c_beta;
-    const T lap = (q10 + qm0 - T(2) * q00) * p.c_lapx + (q01 + q0m - T(2) * q00) * p.c_lapy;
-    const T F = f2d ? f2d[c] : frow[j];
-    const T G = -jac - beta + lap + F;
-    T v = p.b * (q00 + p.dt * G);
-    if (p.a != T(0)) v += p.a * wn[c];
-    wout[c] = v;
-}
 
 // Two-layer stage (Section 2.2, Eq. ge-non with Q_i = q_i - y):
 //   G_1 = -J(psi_1, Q_1) - J(psi_1, y) + A lap w_1 + amp sin(2 pi y)
@@ -149,16 +114,6 @@ __global__ void prolong_kernel(const T* __restrict__ coarse, int ldc,
 }
 
 }  // namespace
-
-template <typename T>
-cudaError_t launch_fine_stage(const T* psi, const T* w, const T* wn, T* wout,
-                              const T* frow, const T* f2d,
-                              const StageParams<T>& p, cudaStream_t s) {
-    const dim3 block(32, 8);
-    const dim3 grid((p.nx - 1 + 31) / 32, (p.ny - 1 + 7) / 8);
-    fine_stage_kernel<T><<<grid, block, 0, s>>>(psi, w, wn, wout, frow, f2d, p);
-    return cudaGetLastError();
-}
 
 template <typename T>
 cudaError_t launch_fine_stage2(const T* psi1, const T* psi2, const T* q1,
@@ -504,9 +459,6 @@ cudaError_t copy_out(void* dense, const void* padded, int ld, int nxm1, int nym1
 }
 
 #define QG_INST(T)                                                                  \
-    template cudaError_t launch_fine_stage<T>(const T*, const T*, const T*, T*,     \
-                                              const T*, const T*,                   \
-                                              const StageParams<T>&, cudaStream_t); \
     template cudaError_t launch_fine_stage2<T>(const T*, const T*, const T*,        \
                                                const T*, const T*, const T*, T*,    \
                                                T*, const T*,                        \
