@@ -66,7 +66,7 @@ struct LevelTables {
 struct MGPlan {
     int nl = 0, tail = 0;
     std::vector<int> mx, my, ld;
-    std::vector<void*> psi, rhs;
+    std::vector<void*> psi, psi2, rhs;
 };
 
 }  // namespace
@@ -488,22 +488,25 @@ qg_status get_mg(qg_ctx* h, int mx, int my, const MGPlan** out) {
         if ((x < y ? x : y) <= 2) break;
     }
     p.nl = (int)p.mx.size();
-    // the tail: the longest run of coarsest grids that fits one CTA's shared
-    // memory (at least the coarsest grid itself)
+    // the tail: the coarsest grids, up to the size below which one CTA's
+    // phases (a barrier each) are shorter than two launches: 32 x 64 nodes;
+    // in FP64, where one SM's units are that few, 16 x 32
+    const long tail_nodes = h->esz == 8 ? 512 : 2048;
     p.tail = p.nl - 1;
     while (p.tail > 0 && p.nl - p.tail < kMaxTail &&
-           mg_tail_smem(&p.mx[p.tail - 1], &p.my[p.tail - 1], p.nl - p.tail + 1, h->esz) <=
-               160 * 1024)
+           (long)p.mx[p.tail - 1] * p.my[p.tail - 1] <= tail_nodes)
         --p.tail;
     if (mg_reserve_tail_smem(mg_tail_smem(&p.mx[p.tail], &p.my[p.tail], p.nl - p.tail, h->esz),
                              h->esz) != cudaSuccess)
         return QG_ERR_CUDA;
     p.psi.assign(p.nl, nullptr);
+    p.psi2.assign(p.nl, nullptr);
     p.rhs.assign(p.nl, nullptr);
     for (int k = 0; k < p.nl; ++k) {
         const size_t bytes = (size_t)(p.my[k] + 1) * p.ld[k] * h->esz;
         qg_status s = dev_alloc(h, &p.rhs[k], bytes);
         if (s == QG_OK && k > 0) s = dev_alloc(h, &p.psi[k], bytes);
+        if (s == QG_OK && k < p.tail) s = dev_alloc(h, &p.psi2[k], bytes);
         if (s != QG_OK) return s;
     }
     auto r = h->mg.emplace(key, std::move(p));
@@ -534,6 +537,7 @@ qg_status mg_solve_level(qg_ctx* h, const LevelTables& t, const void* in, int np
     double dx = t.dxc, dy = t.dyc;
     for (int k = 0; k < mp->nl; ++k, dx *= 2, dy *= 2) {
         lv[k].psi = k == 0 ? static_cast<T*>(out) : static_cast<T*>(mp->psi[k]);
+        lv[k].psi2 = static_cast<T*>(mp->psi2[k]);
         lv[k].rhs_w = static_cast<T*>(mp->rhs[k]);
         lv[k].rhs = lv[k].rhs_w;
         lv[k].mx = mp->mx[k];

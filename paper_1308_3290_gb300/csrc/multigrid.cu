@@ -17,9 +17,19 @@
 //   - two more sweeps.
 // Grids are halved until the shorter side has 2 intervals; there the
 // unknowns form one line and the 5-point equations a tridiagonal system,
-// solved exactly (Thomas algorithm).  The finest levels are one
-// launch per operation; the levels from `tail` down run in one CTA out of
-// shared memory.
+// solved exactly (Thomas algorithm).
+//
+// The grids are small (512 x 1024: 2 MB a field) and every half sweep depends
+// on the one before, so launches are the bound: one per operation, ten a
+// level, took 146 us a cycle on 512 x 1024.  A level takes two launches
+// instead.  A CTA loads a tile of 32 x 32 nodes with a halo as wide as the half
+// sweeps (and the residual's restriction) reach, and does them all in shared
+// memory; the halo's nodes are updated by every CTA that holds them, from the
+// same values in the same order, so the result is that of the whole-grid
+// sweeps.  The tiles of a launch read one array and write another.  The
+// halo costs 1.9 times the arithmetic on the way down and 1.6 on the way up,
+// which the saved passes over the grid repay on large grids too.  The levels
+// from `tail` down run in one CTA out of shared memory.
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -41,17 +51,17 @@ struct Grid {
 };
 
 // ---- one operation on one grid, for a range of threads ---------------
-// (used by the per-level kernels with the whole launch, and by the tail
-// kernel with the CTA)
+// (the tail kernel's)
 
 template <typename T>
 __device__ __forceinline__ void rb_half(const Grid<T>& g, int color, int tid, int nthr) {
     const int hw = g.mx / 2;                   // points of one colour per row (upper bound)
+    const int lh = 31 - __clz(hw);             // (sides are powers of two)
     const int n = hw * (g.my - 1);
     const T inv = T(1) / (T(2) * (g.cx + g.cy));
     for (int e = tid; e < n; e += nthr) {
-        const int j = 1 + e / hw;
-        const int i = 2 * (e % hw) + (((1 + j) & 1) == color ? 1 : 2);
+        const int j = 1 + (e >> lh);
+        const int i = 2 * (e & (hw - 1)) + (((1 + j) & 1) == color ? 1 : 2);
         if (i > g.mx - 1) continue;
         const long long o = (long long)j * g.ld + i, n = (long long)(g.my + 1) * g.ld;
         if (!(QG_IN(o - g.ld, n, 91) && QG_IN(o + g.ld, n, 91) &&
@@ -79,11 +89,11 @@ __device__ __forceinline__ T residual_at(const Grid<T>& g, int i, int j) {
 template <typename T>
 __device__ __forceinline__ void restrict_residual(const Grid<T>& g, T* cf, T* cpsi, int cmx,
                                                   int cmy, int cld, int tid, int nthr) {
-    const int n = (cmx - 1) * (cmy - 1);
+    const int n = cmx * cmy, lc = 31 - __clz(cmx);   // (sides are powers of two)
     for (int e = tid; e < n; e += nthr) {
-        const int I = 1 + e % (cmx - 1), J = 1 + e / (cmx - 1);
+        const int I = e & (cmx - 1), J = e >> lc;
         const int i = 2 * I, j = 2 * J;
-        if (!QG_IN((long long)J * cld + I, (long long)(cmy + 1) * cld, 94)) continue;
+        if (I < 1 || J < 1 || !QG_IN((long long)J * cld + I, (long long)(cmy + 1) * cld, 94)) continue;
         const T c = residual_at(g, i, j);
         const T ed = residual_at(g, i - 1, j) + residual_at(g, i + 1, j) +
                      residual_at(g, i, j - 1) + residual_at(g, i, j + 1);
@@ -98,12 +108,13 @@ __device__ __forceinline__ void restrict_residual(const Grid<T>& g, T* cf, T* cp
 template <typename T>
 __device__ __forceinline__ void prolong_add(const Grid<T>& g, const T* cpsi, int cld, int tid,
                                             int nthr) {
-    const int n = (g.mx - 1) * (g.my - 1);
+    const int n = g.mx * g.my, lx = 31 - __clz(g.mx);
     for (int e = tid; e < n; e += nthr) {
-        const int i = 1 + e % (g.mx - 1), j = 1 + e / (g.mx - 1);
+        const int i = e & (g.mx - 1), j = e >> lx;
         const int I = i >> 1, J = j >> 1;
         const long long cn = (long long)((g.my >> 1) + 1) * cld;
-        if (!(QG_IN((long long)J * cld + I, cn, 95) && QG_IN((long long)(J + 1) * cld + I + 1, cn, 95) &&
+        (void)cn;
+        if (i < 1 || j < 1 || !(QG_IN((long long)J * cld + I, cn, 95) && QG_IN((long long)(J + 1) * cld + I + 1, cn, 95) &&
               QG_IN((long long)j * g.ld + i, (long long)(g.my + 1) * g.ld, 96)))
             continue;
         const T* c = cpsi + (size_t)J * cld + I;
@@ -148,30 +159,193 @@ __device__ void line_solve(const Grid<T>& g) {
 
 // ---- per-level kernels ---------------------------------------------------
 
-template <typename T>
-__global__ void __launch_bounds__(256) mg_rb_kernel(Grid<T> g, int color) {
-    rb_half(g, color, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+constexpr int TW = 32;                        // tile sides
+constexpr int kThreads = 256;
+
+// A tile and its halo of HALO nodes in shared memory: local node (c, r) is
+// node (x0 - HALO + c, y0 - HALO + r).
+template <typename T, int HALO>
+struct Patch {
+    static constexpr int W = TW + 2 * HALO, P = W + 1;   // side, pitch
+    T psi[W * P], rhs[W * P];
+};
+
+// SWEEPS red-black sweeps of the patch: each half sweep updates the nodes one
+// node further in than the last, so that the tile (and what the caller needs
+// around it) sees none of the stale border.
+template <typename T, int HALO, int SWEEPS>
+__device__ __forceinline__ void patch_sweeps(Patch<T, HALO>& s, const Grid<T>& g, int x0, int y0) {
+    using Q = Patch<T, HALO>;
+    constexpr int W = Q::W, HW = W / 2, P = Q::P;
+    const T inv = T(1) / (T(2) * (g.cx + g.cy));
+    constexpr int ITER = (W * HW + kThreads - 1) / kThreads;
+#pragma unroll
+    for (int h = 1; h <= 2 * SWEEPS; ++h) {
+        const int color = (h - 1) & 1;
+        // (the nodes of a colour do not depend on one another: all loads first)
+        T v[ITER];
+        bool ok[ITER];
+        int at[ITER];
+#pragma unroll
+        for (int k = 0; k < ITER; ++k) {
+            const int e = threadIdx.x + k * kThreads;
+            const int r = e / HW, j = y0 - HALO + r;
+            // nodes with (i + j) mod 2 == color (x0, y0 and HALO are even)
+            const int c = 2 * (e - r * HW) + ((r + color) & 1), i = x0 - HALO + c;
+            ok[k] = r >= h && r < W - h && c >= h && c < W - h && i >= 1 && j >= 1 &&
+                    i <= g.mx - 1 && j <= g.my - 1 && QG_IN(r * P + c - P, W * P, 91) &&
+                    QG_IN(r * P + c + P, W * P, 91);
+            at[k] = r * P + c;
+            if (ok[k]) {
+                const T* p = s.psi + at[k];
+                v[k] = (g.cx * (p[-1] + p[1]) + g.cy * (p[-P] + p[P]) - s.rhs[at[k]]) * inv;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < ITER; ++k)
+            if (ok[k]) s.psi[at[k]] = v[k];
+        __syncthreads();
+    }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) mg_restrict_kernel(Grid<T> g, T* cf, T* cpsi, int cmx,
-                                                          int cmy, int cld) {
-    restrict_residual(g, cf, cpsi, cmx, cmy, cld, blockIdx.x * blockDim.x + threadIdx.x,
-                      gridDim.x * blockDim.x);
+template <typename T, int HALO>
+__device__ __forceinline__ T patch_residual(const Patch<T, HALO>& s, const Grid<T>& g, int x0,
+                                            int y0, int c, int r) {
+    constexpr int P = Patch<T, HALO>::P, W = Patch<T, HALO>::W;
+    const int i = x0 - HALO + c, j = y0 - HALO + r;
+    if (i < 1 || j < 1 || i > g.mx - 1 || j > g.my - 1) return T(0);
+    if (!(QG_IN(r * P + c - P, W * P, 93) && QG_IN(r * P + c + P, W * P, 93)))
+        return T(0);
+    const T* p = s.psi + r * P + c;
+    const T lap = g.cx * (p[-1] + p[1] - T(2) * p[0]) + g.cy * (p[-P] + p[P] - T(2) * p[0]);
+    return s.rhs[r * P + c] - lap;
 }
 
+// Down: the pre-smoothing sweeps of g (from zero when `zero`, else from
+// g.psi) -> out, and the residual's restriction -> cf.
 template <typename T>
-__global__ void __launch_bounds__(256) mg_prolong_kernel(Grid<T> g, const T* cpsi, int cld) {
-    prolong_add(g, cpsi, cld, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+__global__ void __launch_bounds__(kThreads)
+mg_down_kernel(Grid<T> g, int zero, T* out, T* cf, int cmx, int cmy, int cld) {
+    // 2 kPre half sweeps, the residual beside the tile, its stencil
+    constexpr int HALO = 2 * kPre + 2;
+    using Q = Patch<T, HALO>;
+    __shared__ Q s;
+    const int x0 = blockIdx.x * TW, y0 = blockIdx.y * TW;
+    pdl_wait();
+    pdl_trigger();
+    constexpr int ITER = (Q::W * Q::W + kThreads - 1) / kThreads;
+    T pv[ITER], fv[ITER];
+#pragma unroll
+    for (int k = 0; k < ITER; ++k) {
+        const int e = threadIdx.x + k * kThreads;
+        const int r = e / Q::W, c = e - r * Q::W, i = x0 - HALO + c, j = y0 - HALO + r;
+        const bool in = r < Q::W && i >= 1 && j >= 1 && i <= g.mx - 1 && j <= g.my - 1 &&
+                        QG_IN((long long)j * g.ld + i, (long long)(g.my + 1) * g.ld, 92) &&
+                        QG_IN((long long)j * g.ldr + i, (long long)(g.my + 1) * g.ldr, 92);
+        pv[k] = in && !zero ? g.psi[(size_t)j * g.ld + i] : T(0);
+        fv[k] = in ? g.rhs[(size_t)j * g.ldr + i] : T(0);
+    }
+#pragma unroll
+    for (int k = 0; k < ITER; ++k) {
+        const int e = threadIdx.x + k * kThreads;
+        const int r = e / Q::W, c = e - r * Q::W;
+        if (r < Q::W) {
+            s.psi[r * Q::P + c] = pv[k];
+            s.rhs[r * Q::P + c] = fv[k];
+        }
+    }
+    __syncthreads();
+    patch_sweeps<T, HALO, kPre>(s, g, x0, y0);
+    for (int e = threadIdx.x; e < TW * TW; e += kThreads) {
+        const int c = e % TW, r = e / TW, i = x0 + c, j = y0 + r;
+        if (i >= 1 && j >= 1 && i <= g.mx - 1 && j <= g.my - 1 &&
+            QG_IN((long long)j * g.ld + i, (long long)(g.my + 1) * g.ld, 96))
+            out[(size_t)j * g.ld + i] = s.psi[(r + HALO) * Q::P + c + HALO];
+    }
+    for (int e = threadIdx.x; e < TW * TW / 4; e += kThreads) {
+        const int I = x0 / 2 + e % (TW / 2), J = y0 / 2 + e / (TW / 2);
+        if (I < 1 || J < 1 || I > cmx - 1 || J > cmy - 1 ||
+            !QG_IN((long long)J * cld + I, (long long)(cmy + 1) * cld, 94))
+            continue;
+        const int c = 2 * I - x0 + HALO, r = 2 * J - y0 + HALO;
+        auto res = [&](int dc, int dr) { return patch_residual<T, HALO>(s, g, x0, y0, c + dc, r + dr); };
+        const T ed = res(-1, 0) + res(1, 0) + res(0, -1) + res(0, 1);
+        const T co = res(-1, -1) + res(1, -1) + res(-1, 1) + res(1, 1);
+        cf[(size_t)J * cld + I] = (T(4) * res(0, 0) + T(2) * ed + co) * T(0.0625);
+    }
+}
+
+// Up: g.psi + P(coarse psi), the post-smoothing sweeps -> out.
+template <typename T>
+__global__ void __launch_bounds__(kThreads)
+mg_up_kernel(Grid<T> g, T* out, const T* cpsi, int cld) {
+    constexpr int HALO = 2 * kPost;
+    using Q = Patch<T, HALO>;
+    __shared__ Q s;
+    const int x0 = blockIdx.x * TW, y0 = blockIdx.y * TW;
+    pdl_wait();
+    pdl_trigger();
+    constexpr int ITER = (Q::W * Q::W + kThreads - 1) / kThreads;
+    T q[ITER][4], pv[ITER], fv[ITER];
+#pragma unroll
+    for (int k = 0; k < ITER; ++k) {
+        const int e = threadIdx.x + k * kThreads;
+        const int r = e / Q::W, c = e - r * Q::W, i = x0 - HALO + c, j = y0 - HALO + r;
+        const long long cn = (long long)((g.my >> 1) + 1) * cld;
+        (void)cn;
+        const int I = i >> 1, J = j >> 1;
+        const bool in = r < Q::W && i >= 1 && j >= 1 && i <= g.mx - 1 && j <= g.my - 1 &&
+                        QG_IN((long long)(J + 1) * cld + I + 1, cn, 95) &&
+                        QG_IN((long long)j * g.ld + i, (long long)(g.my + 1) * g.ld, 92);
+        // the four elliptic nodes around (zero walls)
+        const T* cq = cpsi + (in ? (size_t)J * cld + I : 0);
+        q[k][0] = in ? cq[0] : T(0);
+        q[k][1] = in ? cq[1] : T(0);
+        q[k][2] = in ? cq[cld] : T(0);
+        q[k][3] = in ? cq[cld + 1] : T(0);
+        pv[k] = in ? g.psi[(size_t)j * g.ld + i] : T(0);
+        fv[k] = in ? g.rhs[(size_t)j * g.ldr + i] : T(0);
+    }
+#pragma unroll
+    for (int k = 0; k < ITER; ++k) {
+        const int e = threadIdx.x + k * kThreads;
+        const int r = e / Q::W, c = e - r * Q::W;   // (x0, y0 and HALO are even)
+        const T lo = (c & 1) ? T(0.5) * (q[k][0] + q[k][1]) : q[k][0];
+        const T hi = (c & 1) ? T(0.5) * (q[k][2] + q[k][3]) : q[k][2];
+        pv[k] += (r & 1) ? T(0.5) * (lo + hi) : lo;
+    }
+#pragma unroll
+    for (int k = 0; k < ITER; ++k) {
+        const int e = threadIdx.x + k * kThreads;
+        const int r = e / Q::W, c = e - r * Q::W;
+        if (r < Q::W) {
+            s.psi[r * Q::P + c] = pv[k];
+            s.rhs[r * Q::P + c] = fv[k];
+        }
+    }
+    __syncthreads();
+    patch_sweeps<T, HALO, kPost>(s, g, x0, y0);
+    for (int e = threadIdx.x; e < TW * TW; e += kThreads) {
+        const int c = e % TW, r = e / TW, i = x0 + c, j = y0 + r;
+        if (i >= 1 && j >= 1 && i <= g.mx - 1 && j <= g.my - 1 &&
+            QG_IN((long long)j * g.ld + i, (long long)(g.my + 1) * g.ld, 96))
+            out[(size_t)j * g.ld + i] = s.psi[(r + HALO) * Q::P + c + HALO];
+    }
 }
 
 // rhs0 = P0 + P1 + ... (the restriction's partial planes, in that order),
 // psi0 = 0 when `zero`
 template <typename T>
 __global__ void __launch_bounds__(256) mg_sum_kernel(MGSumParams<T> q) {
-    const int n = (q.mx - 1) * (q.my - 1);
+    const int n = q.mx * q.my, lx = 31 - __clz(q.mx);
+    pdl_wait();
+    pdl_trigger();
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-        const int i = 1 + e % (q.mx - 1), j = 1 + e / (q.mx - 1);
+        const int i = e & (q.mx - 1), j = e >> lx;
+        if (i < 1 || j < 1) continue;
         const size_t o = (size_t)j * q.ld_in + i;
         T v = q.in[0][o];
         for (int k = 1; k < q.nin; ++k) v = v + q.in[k][o];
@@ -180,11 +354,13 @@ __global__ void __launch_bounds__(256) mg_sum_kernel(MGSumParams<T> q) {
     }
 }
 
+constexpr int kTailThreads = 512;
+
 // ---- the tail: levels t..C in one CTA, out of shared memory -------------
-// On entry psi_t (global) holds the initial guess and rhs_t (global) the
+// On entry psi_t (global) holds the initial guess (zero: a.zero) and rhs_t (global) the
 // right-hand side; one V-cycle over levels t..C; psi_t is written back.
 template <typename T>
-__global__ void __launch_bounds__(512) mg_tail_kernel(MGTail<T> a) {
+__global__ void __launch_bounds__(kTailThreads) mg_tail_kernel(MGTail<T> a) {
     extern __shared__ __align__(16) unsigned char smem[];
     T* base = reinterpret_cast<T*>(smem);
     const int tid = threadIdx.x, nthr = blockDim.x;
@@ -214,16 +390,31 @@ __global__ void __launch_bounds__(512) mg_tail_kernel(MGTail<T> a) {
 #endif
     for (size_t e = tid; e < off; e += nthr) base[e] = T(0);
     __syncthreads();
+    pdl_wait();
+    pdl_trigger();
     {
-        const int n = (a.mx[0] + 1) * (a.my[0] + 1);
+        const int n = a.mx[0] * a.my[0], lx = 31 - __clz(a.mx[0]), ld0 = g[0].ld;
         T* rhs0 = const_cast<T*>(g[0].rhs);
-        for (int e = tid; e < n; e += nthr) {
-            const int i = e % (a.mx[0] + 1), j = e / (a.mx[0] + 1);
-            const bool in = i >= 1 && j >= 1 && i <= a.mx[0] - 1 && j <= a.my[0] - 1 &&
-                            QG_IN((long long)j * a.ld + i, (long long)(a.my[0] + 1) * a.ld, 98) &&
-                            QG_IN((long long)j * a.ldr + i, (long long)(a.my[0] + 1) * a.ldr, 98);
-            g[0].psi[e] = in ? a.psi[(size_t)j * a.ld + i] : T(0);
-            rhs0[e] = in ? a.rhs[(size_t)j * a.ldr + i] : T(0);
+        constexpr int U = 4;                      // loads in flight
+        for (int e0 = tid; e0 < n; e0 += U * nthr) {
+            T pv[U], fv[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int e = e0 + u * nthr, i = e & (a.mx[0] - 1), j = e >> lx;
+                const bool in = e < n && i >= 1 && j >= 1 &&
+                                QG_IN((long long)j * a.ld + i, (long long)(a.my[0] + 1) * a.ld, 98) &&
+                                QG_IN((long long)j * a.ldr + i, (long long)(a.my[0] + 1) * a.ldr, 98);
+                pv[u] = in && !a.zero ? a.psi[(size_t)j * a.ld + i] : T(0);
+                fv[u] = in ? a.rhs[(size_t)j * a.ldr + i] : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int e = e0 + u * nthr, i = e & (a.mx[0] - 1), j = e >> lx;
+                if (e < n) {
+                    g[0].psi[j * ld0 + i] = pv[u];
+                    rhs0[j * ld0 + i] = fv[u];
+                }
+            }
         }
     }
     __syncthreads();
@@ -248,9 +439,10 @@ __global__ void __launch_bounds__(512) mg_tail_kernel(MGTail<T> a) {
                 __syncthreads();
             }
     }
-    const int n = (a.mx[0] - 1) * (a.my[0] - 1);
+    const int n = a.mx[0] * a.my[0], lx = 31 - __clz(a.mx[0]);
     for (int e = tid; e < n; e += nthr) {
-        const int i = 1 + e % (a.mx[0] - 1), j = 1 + e / (a.mx[0] - 1);
+        const int i = e & (a.mx[0] - 1), j = e >> lx;
+        if (i < 1 || j < 1) continue;
         if (!QG_IN((long long)j * a.ld + i, (long long)(a.my[0] + 1) * a.ld, 99)) continue;
         a.psi[(size_t)j * a.ld + i] = g[0].psi[(size_t)j * g[0].ld + i];
     }
@@ -283,7 +475,7 @@ cudaError_t mg_reserve_tail_smem(size_t bytes, size_t esz) {
     return e;
 }
 
-int mg_cycle_launches(int tail) { return tail * (2 * kPre + 2 * kPost + 2) + 1; }
+int mg_cycle_launches(int tail) { return 2 * tail + 1; }
 
 size_t mg_tail_smem(const int* mx, const int* my, int n, size_t esz) {
     size_t s = 0;
@@ -291,19 +483,37 @@ size_t mg_tail_smem(const int* mx, const int* my, int n, size_t esz) {
     return s;
 }
 
-template <typename T>
-cudaError_t launch_mg_sum(const MGSumParams<T>& q, cudaStream_t s) {
-    mg_sum_kernel<T><<<blocks_for((long)(q.mx - 1) * (q.my - 1)), 256, 0, s>>>(q);
-    return cudaGetLastError();
+// A launch that depends programmatically on the one before it.
+template <typename... P, typename... A>
+static cudaError_t launch(void (*k)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s,
+                          const A&... a) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, P(a)...);
 }
 
-// One V-cycle.  lv[0..nl): the grids (psi, rhs, sizes, pitches, 1/dx^2,
-// 1/dy^2); the levels from `tail` on are the tail's.
+template <typename T>
+cudaError_t launch_mg_sum(const MGSumParams<T>& q, cudaStream_t s) {
+    return launch(mg_sum_kernel<T>, dim3(blocks_for((long)q.mx * q.my)), 256, 0, s, q);
+}
+
+// One V-cycle.  lv[0..nl): the grids (psi, psi2, rhs, sizes, pitches, 1/dx^2,
+// 1/dy^2); the levels from `tail` on are the tail's.  Level 0 starts from its
+// psi, the others from zero; every level's result is in psi (its smoothed
+// state on the way down in psi2).
 template <typename T>
 cudaError_t launch_mg_cycle(const MGLevelDesc<T>* lv, int nl, int tail, cudaStream_t s) {
-    auto grid = [&](int k) {
+    auto grid = [&](int k, T* psi) {
         Grid<T> g;
-        g.psi = lv[k].psi;
+        g.psi = psi;
         g.rhs = lv[k].rhs;
         g.mx = lv[k].mx;
         g.my = lv[k].my;
@@ -313,41 +523,31 @@ cudaError_t launch_mg_cycle(const MGLevelDesc<T>* lv, int nl, int tail, cudaStre
         g.cy = lv[k].cy;
         return g;
     };
-    for (int k = 0; k < tail; ++k) {
-        const Grid<T> g = grid(k);
-        const int nb = blocks_for((long)(g.mx / 2) * (g.my - 1));
-        for (int p = 0; p < kPre; ++p)
-            for (int c = 0; c < 2; ++c) mg_rb_kernel<T><<<nb, 256, 0, s>>>(g, c);
-        mg_restrict_kernel<T><<<blocks_for((long)(lv[k + 1].mx - 1) * (lv[k + 1].my - 1)), 256, 0,
-                                s>>>(g, lv[k + 1].rhs_w, lv[k + 1].psi, lv[k + 1].mx,
-                                     lv[k + 1].my, lv[k + 1].ld);
+    auto tiles = [&](int k) { return dim3((lv[k].mx + TW - 1) / TW, (lv[k].my + TW - 1) / TW); };
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < tail && e == cudaSuccess; ++k)
+        e = launch(mg_down_kernel<T>, tiles(k), kThreads, 0, s, grid(k, lv[k].psi), k > 0 ? 1 : 0,
+                   lv[k].psi2, lv[k + 1].rhs_w, lv[k + 1].mx, lv[k + 1].my, lv[k + 1].ld);
+    if (e != cudaSuccess) return e;
+    MGTail<T> a = {};
+    a.n = nl - tail;
+    if (a.n > kMaxTail) return cudaErrorInvalidValue;
+    for (int k = 0; k < a.n; ++k) {
+        a.mx[k] = lv[tail + k].mx;
+        a.my[k] = lv[tail + k].my;
+        a.cx[k] = lv[tail + k].cx;
+        a.cy[k] = lv[tail + k].cy;
     }
-    {
-        MGTail<T> a = {};
-        a.n = nl - tail;
-        if (a.n > kMaxTail) return cudaErrorInvalidValue;
-        for (int k = 0; k < a.n; ++k) {
-            a.mx[k] = lv[tail + k].mx;
-            a.my[k] = lv[tail + k].my;
-            a.cx[k] = lv[tail + k].cx;
-            a.cy[k] = lv[tail + k].cy;
-        }
-        a.psi = lv[tail].psi;
-        a.rhs = lv[tail].rhs;
-        a.ld = lv[tail].ld;
-        a.ldr = lv[tail].ldr;
-        const size_t sm = mg_tail_smem(a.mx, a.my, a.n, sizeof(T));
-        mg_tail_kernel<T><<<1, 512, sm, s>>>(a);
-    }
-    for (int k = tail - 1; k >= 0; --k) {
-        const Grid<T> g = grid(k);
-        mg_prolong_kernel<T><<<blocks_for((long)(g.mx - 1) * (g.my - 1)), 256, 0, s>>>(
-            g, lv[k + 1].psi, lv[k + 1].ld);
-        const int nb = blocks_for((long)(g.mx / 2) * (g.my - 1));
-        for (int p = 0; p < kPost; ++p)
-            for (int c = 0; c < 2; ++c) mg_rb_kernel<T><<<nb, 256, 0, s>>>(g, c);
-    }
-    return cudaGetLastError();
+    a.psi = lv[tail].psi;
+    a.rhs = lv[tail].rhs;
+    a.ld = lv[tail].ld;
+    a.ldr = lv[tail].ldr;
+    a.zero = tail > 0 ? 1 : 0;
+    e = launch(mg_tail_kernel<T>, dim3(1), kTailThreads, mg_tail_smem(a.mx, a.my, a.n, sizeof(T)), s, a);
+    for (int k = tail - 1; k >= 0 && e == cudaSuccess; --k)
+        e = launch(mg_up_kernel<T>, tiles(k), kThreads, 0, s, grid(k, lv[k].psi2), lv[k].psi,
+                   lv[k + 1].psi, lv[k + 1].ld);
+    return e;
 }
 
 QG_BOUNDS_QUERY(bounds_site_mg)

@@ -350,6 +350,7 @@ constexpr int kMaxTail = 14;          // levels the one-CTA tail can hold
 template <typename T>
 struct MGLevelDesc {                  // one grid of the hierarchy
     T* psi;                           // (my+1) rows of pitch ld, zero walls
+    T* psi2;                          // another one (levels above the tail)
     const T* rhs;                     // right-hand side, pitch ldr
     T* rhs_w;                         // the same, writable (levels >= 1)
     int mx, my, ld, ldr;
@@ -363,6 +364,7 @@ struct MGTail {                       // levels handled by one CTA in shared mem
     T* psi;                           // first tail level (global): guess in, result out
     const T* rhs;
     int ld, ldr;
+    int zero;                         // 1: the guess is zero
 };
 template <typename T>
 struct MGSumParams {                  // rhs = in[0] + in[1] + ..., psi = 0 if zero
