@@ -136,6 +136,13 @@ struct qg_ctx {
     double* hout = nullptr;        // pinned host copy of the 5 diagnostics
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t gexec = nullptr;
+    // the step captured with the time means switched the other way (null: not
+    // yet), swapped in when they are: a window of means costs no capture
+    struct {
+        cudaGraph_t graph = nullptr;
+        cudaGraphExec_t gexec = nullptr;
+        int64_t kernels = 0;
+    } parked;
     qg_status latched = QG_OK;
     std::vector<void*> allocs;
     cudaMemPool_t pool = nullptr;  // scratch of the stand-alone calls (scratch_alloc)
@@ -1079,6 +1086,8 @@ qg_status stage_fused(qg_ctx* h, int s_idx, cudaStream_t s) {
     const LevelTables* t = nullptr;
     qg_status st = get_level(h, h->levels, &t);
     if (st != QG_OK) return fail(h, st);
+    // (before the solve, off the chain of dependent launches)
+    if (s_idx == 0 && h->cfl > 0.0) QG_TRY(cudaMemsetAsync(h->dclock, 0, sizeof(double), s));
     if (h->levels == 0) {
         st = solve_level<T>(h, *t, win, h->ct, h->ld_t, h->plane_t, h->cw, h->psi,
                             h->plane_f, s, 1);
@@ -1087,12 +1096,28 @@ qg_status stage_fused(qg_ctx* h, int s_idx, cudaStream_t s) {
                             h->plane_c, s, 4);
     }
     if (st != QG_OK) return st;
-    if (h->stats && s_idx == 0) {
+    if (s_idx == 0 && (h->stats || h->cfl > 0.0)) {
         const bool fine = h->levels == 0;
-        QG_TRY(launch_accumulate<T>(h->stat_acc, static_cast<const T*>(fine ? h->psi : h->cpsi),
-                                    (fine ? h->plane_f : h->plane_c) * h->layers, s));
-        QG_TRY(launch_accumulate<T>(h->stat_acc_w, static_cast<const T*>(h->w[0]),
-                                    h->plane_f * h->layers, s));
+        FirstStage<T> q = {};
+        q.psi = static_cast<const T*>(fine ? h->psi : h->cpsi);
+        q.ldp = fine ? h->ldf : t->ldc;
+        q.n_psi = (int)((fine ? h->plane_f : h->plane_c) * h->layers);
+        q.w = static_cast<const T*>(h->w[0]);
+        q.n_w = (int)(h->plane_f * h->layers);
+        q.nx = h->nx;
+        q.ny = h->ny;
+        q.inv2dx = 0.5 / h->dx;
+        q.inv2dy = 0.5 / h->dy;
+        q.acc_psi = h->stats ? h->stat_acc : nullptr;
+        q.acc_w = h->stats ? h->stat_acc_w : nullptr;
+        if (h->cfl > 0.0) {
+            // Eq. dt from psi^n, the streamfunction of this first stage
+            q.umax = reinterpret_cast<unsigned long long*>(h->dclock);
+            KTimer kc(h, s, QG_K_CFL);
+            QG_TRY(launch_first_stage<T>(q, h->levels, s));
+        } else {
+            QG_TRY(launch_first_stage<T>(q, h->levels, s));
+        }
     }
     if (h->layers == 2) return stage_fused2<T>(h, s_idx, *t, s);
     FusedParams<T> p;
@@ -1124,17 +1149,7 @@ qg_status stage_fused(qg_ctx* h, int s_idx, cudaStream_t s) {
     p.dt_cap = h->dt;
     p.clock = h->dclock + 1;
     p.last_stage = s_idx == 2;
-    if (h->cfl > 0.0) {
-        p.umax = reinterpret_cast<const unsigned long long*>(h->dclock);
-        if (s_idx == 0) {
-            // Eq. dt from psi^n, the streamfunction of this first stage
-            QG_TRY(cudaMemsetAsync(h->dclock, 0, sizeof(double), s));
-            KTimer kc(h, s, QG_K_CFL);
-            QG_TRY(launch_cfl_max<T>(static_cast<const T*>(p.psi), p.ldp, h->nx, h->ny,
-                                     h->levels, h->dx, h->dy,
-                                     reinterpret_cast<unsigned long long*>(h->dclock), s));
-        }
-    }
+    if (h->cfl > 0.0) p.umax = reinterpret_cast<const unsigned long long*>(h->dclock);
     FineMaps m;
     m.w = h->tm_halo[s_idx][0];
     m.wn = h->tm_int[0][0];
@@ -1185,10 +1200,12 @@ void drop_graph(qg_ctx* h) {
         *r = Replay();
     }
     ++h->graph_gen;
-    if (h->gexec) cudaGraphExecDestroy(h->gexec);
-    if (h->graph) cudaGraphDestroy(h->graph);
-    h->gexec = nullptr;
-    h->graph = nullptr;
+    for (cudaGraphExec_t x : {h->gexec, h->parked.gexec})
+        if (x) cudaGraphExecDestroy(x);
+    for (cudaGraph_t g : {h->graph, h->parked.graph})
+        if (g) cudaGraphDestroy(g);
+    h->gexec = h->parked.gexec = nullptr;
+    h->graph = h->parked.graph = nullptr;
 }
 
 qg_status build_graph(qg_ctx* h) {
@@ -1781,6 +1798,20 @@ qg_status qg_get_time(qg_handle h, double* t, double* dt_last) {
     return QG_OK;
 }
 
+// Switch the time means on or off, and with them the captured step.
+static void switch_stats(qg_ctx* h, bool on) {
+    if (h->stats == on) return;
+    if (h->timing) {
+        drop_graph(h);   // (its events belong to the step being timed)
+    } else {
+        std::swap(h->graph, h->parked.graph);
+        std::swap(h->gexec, h->parked.gexec);
+        std::swap(h->kernels_per_step, h->parked.kernels);
+        ++h->graph_gen;
+    }
+    h->stats = on;
+}
+
 qg_status qg_stats_begin(qg_handle h) {
     if (!h) return QG_ERR_ARG;
     if (h->tape) return QG_ERR_UNSUPPORTED;
@@ -1799,11 +1830,7 @@ qg_status qg_stats_begin(qg_handle h) {
     QG_TRY(cudaMemsetAsync(h->stat_acc, 0, n * sizeof(double), h->stream));
     QG_TRY(cudaMemsetAsync(h->stat_acc_w, 0, nw * sizeof(double), h->stream));
     h->stat_count = 0;
-    if (!h->stats) {
-        QG_TRY(cudaStreamSynchronize(h->stream));
-        drop_graph(h);
-        h->stats = true;
-    }
+    switch_stats(h, true);
     return QG_OK;
 }
 
@@ -1852,11 +1879,7 @@ qg_status qg_stats_mean_q(qg_handle h, void* q_mean, int layer, int64_t* count) 
 
 qg_status qg_stats_end(qg_handle h) {
     if (!h) return QG_ERR_ARG;
-    if (h->stats) {
-        QG_TRY(cudaStreamSynchronize(h->stream));
-        drop_graph(h);
-        h->stats = false;
-    }
+    switch_stats(h, false);
     return QG_OK;
 }
 

@@ -243,6 +243,22 @@ struct FusedParams {
     T inv_Ro, k_p, drag;
 };
 
+// What a step's first stage adds after its solve (stencil.cu).
+template <typename T>
+struct FirstStage {
+    const T* psi;                 // elliptic-grid psi (l = 0: fine), pitch ldp, n_psi elements
+    int ldp, n_psi;
+    const T* w;                   // the state, n_w elements
+    int n_w;
+    int nx, ny;
+    double inv2dx, inv2dy;        // 1/(2 dx), 1/(2 dy)
+    unsigned long long* umax;     // launch_cfl_max's, zeroed before, or null
+    double* acc_psi;              // time-mean sums, or null
+    double* acc_w;
+};
+template <typename T>
+cudaError_t launch_first_stage(const FirstStage<T>& q, int levels, cudaStream_t s);
+
 // acc[e] += src[e] for the n elements of a padded plane (FP64 sums).
 template <typename T>
 cudaError_t launch_accumulate(double* acc, const T* src, size_t n, cudaStream_t s);

@@ -192,8 +192,8 @@ __device__ __forceinline__ T prolonged_at(const T* __restrict__ c, int ldc, int 
 // maximum is max-ed into *umax as the bits of a non-negative double (bit
 // order = value order), so the result does not depend on the block order.
 template <typename T, int LV>
-__global__ void cfl_max_kernel(const T* __restrict__ psi, int ldp, int nx, int ny,
-                               double inv2dx, double inv2dy, unsigned long long* umax) {
+__device__ __forceinline__ void cfl_max(const T* __restrict__ psi, int ldp, int nx, int ny,
+                                        double inv2dx, double inv2dy, unsigned long long* umax) {
     constexpr int F = 1 << LV, W = F + 2;
     __shared__ double red[32];
     // maxima of |psi(x+1) - psi(x-1)| and |psi(y+1) - psi(y-1)| in the
@@ -201,10 +201,9 @@ __global__ void cfl_max_kernel(const T* __restrict__ psi, int ldp, int nx, int n
     // scaling by 1/(2 dx), 1/(2 dy) is monotone, so it is applied once
     T ax = T(0), ay = T(0);
     const int mx = nx >> LV, my = ny >> LV;
-    const long ncell = (long)mx * my;
-    for (long e = (long)blockIdx.x * blockDim.x + threadIdx.x; e < ncell;
-         e += (long)gridDim.x * blockDim.x) {
-        const int I = (int)(e % mx), J = (int)(e / mx);
+    const int ncell = mx * my, lmx = 31 - __clz(mx);   // (sides are powers of two)
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < ncell; e += gridDim.x * blockDim.x) {
+        const int I = e & (mx - 1), J = e >> lmx;
         if constexpr (LV == 0) {   // the fine psi itself: one node per thread
             if (I < 1 || J < 1) continue;
             const T* p = psi + (size_t)J * ldp + I;
@@ -270,6 +269,81 @@ __global__ void cfl_max_kernel(const T* __restrict__ psi, int ldp, int nx, int n
     }
 }
 
+template <typename T, int LV>
+__global__ void cfl_max_kernel(const T* psi, int ldp, int nx, int ny, double inv2dx, double inv2dy,
+                               unsigned long long* umax) {
+    cfl_max<T, LV>(psi, ldp, nx, ny, inv2dx, inv2dy, umax);
+}
+
+// acc[e] += src[e], four values a thread and pass (n is a multiple of 4: a
+// padded plane).
+template <typename T>
+__device__ __forceinline__ void accumulate(double* __restrict__ acc, const T* __restrict__ src,
+                                           int n) {
+    for (int e = 4 * (blockIdx.x * blockDim.x + threadIdx.x); e < n; e += 4 * gridDim.x * blockDim.x) {
+        T v[4];
+        if constexpr (sizeof(T) == 4) {
+            const float4 q = *reinterpret_cast<const float4*>(src + e);
+            v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = src[e + k];
+        }
+        double2* a = reinterpret_cast<double2*>(acc + e);
+        double2 a0 = a[0], a1 = a[1];
+        a0.x += (double)v[0];
+        a0.y += (double)v[1];
+        a1.x += (double)v[2];
+        a1.y += (double)v[3];
+        a[0] = a0;
+        a[1] = a1;
+    }
+}
+
+// What a step's first stage adds between its solve and its update: the
+// maximum of Eq. dt (q.umax) and the time means' sums (q.acc_psi, q.acc_w).
+// One launch between two that are chained programmatically: as three
+// launches and a memset of their own they took 30 us of an 82 us step of
+// 1024 x 512, l = 1.
+template <typename T, int LV, bool CFL>
+__global__ void __launch_bounds__(256) first_stage_kernel(FirstStage<T> q) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (q.acc_w) accumulate(q.acc_w, q.w, q.n_w);
+    if (q.acc_psi) accumulate(q.acc_psi, q.psi, q.n_psi);
+    if constexpr (CFL) cfl_max<T, LV>(q.psi, q.ldp, q.nx, q.ny, q.inv2dx, q.inv2dy, q.umax);
+}
+
+template <typename T>
+cudaError_t launch_first_stage(const FirstStage<T>& q, int levels, cudaStream_t s) {
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    long items = q.umax ? (long)(q.nx >> levels) * (q.ny >> levels) : 0;
+    if (q.acc_w && q.n_w / 4 > items) items = q.n_w / 4;
+    if (q.acc_psi && q.n_psi / 4 > items) items = q.n_psi / 4;
+    long blocks = (items + 255) / 256;
+    if (blocks > 8L * nsm) blocks = 8L * nsm;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (!q.umax) return cudaLaunchKernelEx(&cfg, first_stage_kernel<T, 0, false>, q);
+    switch (levels) {
+        case 0: return cudaLaunchKernelEx(&cfg, first_stage_kernel<T, 0, true>, q);
+        case 1: return cudaLaunchKernelEx(&cfg, first_stage_kernel<T, 1, true>, q);
+        case 2: return cudaLaunchKernelEx(&cfg, first_stage_kernel<T, 2, true>, q);
+        case 3: return cudaLaunchKernelEx(&cfg, first_stage_kernel<T, 3, true>, q);
+        case 4: return cudaLaunchKernelEx(&cfg, first_stage_kernel<T, 4, true>, q);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
 template <typename T>
 cudaError_t launch_cfl_max(const T* psi, int ldp, int nx, int ny, int levels, double dx,
                            double dy, unsigned long long* umax, cudaStream_t s) {
@@ -291,10 +365,8 @@ cudaError_t launch_cfl_max(const T* psi, int ldp, int nx, int ny, int levels, do
 }
 
 template <typename T>
-__global__ void accumulate_kernel(double* __restrict__ acc, const T* __restrict__ src, size_t n) {
-    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-         e += (size_t)gridDim.x * blockDim.x)
-        acc[e] += (double)src[e];
+__global__ void __launch_bounds__(256) accumulate_kernel(double* acc, const T* src, int n) {
+    accumulate(acc, src, n);
 }
 
 template <typename T>
@@ -332,9 +404,9 @@ template cudaError_t launch_mean_q_out<double>(double*, const double*, int, doub
 
 template <typename T>
 cudaError_t launch_accumulate(double* acc, const T* src, size_t n, cudaStream_t s) {
-    size_t blocks = (n + 255) / 256;
+    size_t blocks = (n / 4 + 255) / 256;
     if (blocks > 4096) blocks = 4096;
-    accumulate_kernel<T><<<(int)blocks, 256, 0, s>>>(acc, src, n);
+    accumulate_kernel<T><<<(int)blocks, 256, 0, s>>>(acc, src, (int)n);
     return cudaGetLastError();
 }
 
@@ -472,6 +544,7 @@ cudaError_t copy_out(void* dense, const void* padded, int ld, int nxm1, int nym1
     template cudaError_t launch_prolong_dense<T>(const T*, T*, int, int, int, cudaStream_t); \
     template cudaError_t launch_cfl_max<T>(const T*, int, int, int, int, double,     \
                                            double, unsigned long long*, cudaStream_t); \
+    template cudaError_t launch_first_stage<T>(const FirstStage<T>&, int, cudaStream_t); \
     template cudaError_t launch_accumulate<T>(double*, const T*, size_t, cudaStream_t); \
     template cudaError_t launch_mean_out<T>(T*, const double*, int, double, int, int,  \
                                             int, cudaStream_t);
