@@ -409,6 +409,8 @@ qg_status get_level(qg_ctx* h, int lv, const LevelTables** out) {
             }
         }
         half_lam(t.my, ly.data(), v.data() + 2 * (nx + ny));
+        // divided by the solve's scale (2/mx)(2/my)/16, a power of two
+        for (size_t k = 0; k < nl; ++k) v[2 * (nx + ny) + k] *= 4.0 * t.mx * t.my;
         s = upload_real(h, &t.htx, v);
         t.hty = static_cast<char*>(t.htx) + 2 * nx * h->esz;
         t.lamyr = static_cast<char*>(t.htx) + 2 * (nx + ny) * h->esz;

@@ -74,7 +74,7 @@ struct SolveParams {
     const typename Cx<T>::type* pty;   //   2 mx and 2 my (see pass_table_size)
     const typename Cx<T>::type* htx;   // engine 50: half_table(2 mx) and
     const typename Cx<T>::type* hty;   //   half_table(2 my)
-    const T* lamyr;                     // engine 50: lamy in its rows' order (half_lam)
+    const T* lamyr;                     // engine 50: lamy / (scale / 16) in its rows' order (half_lam)
     const T* dsx;                       // engine 42: dense_table(mx) and
     const T* dsy;                       //   dense_table(my)
     const T* lamx;                      // (2 cos(pi k/mx) - 2)/dx^2, k = 0..mx

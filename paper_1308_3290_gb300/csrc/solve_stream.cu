@@ -185,6 +185,15 @@ __device__ __forceinline__ int row_k(int j, int i) {
     }
 }
 
+// Its part that does not depend on the thread: k = 0 and k = G/2 (the walls of
+// row 0) lie at j = 0 of the registers whose part is 0 and G/2.
+template <int LG>
+__host__ __device__ constexpr int row_k0(int i) {
+    using Q = Half<LG>;
+    return Q::HC == 1 ? (i / Q::H) * Q::H + 16 * (i % Q::H)
+                      : 16 * ((Q::H / 16) * (i >> 2) + Q::HB * (i & 3));
+}
+
 // Whether that index is below G/2, the same for every thread.
 template <int LG>
 __host__ __device__ constexpr bool row_low(int i) {
@@ -320,6 +329,7 @@ __device__ __forceinline__ void load_rhs(const SolveParams<T>& P, const T* const
                                          const T* const (&ib)[4], int ra, int rb, bool va, bool vb,
                                          int t, Cplx<T> (&v)[16]) {
     using Q = Half<LG>;
+    // (a row that does not exist reads row 0, a wall: zeros)
     const int oa = (va ? ra : 0) * P.ld, ob = (vb ? rb : 0) * P.ld;
     const bool cx = P.nin > 1 && (t & (P.part_px - 1)) == 0;
     const bool ya = P.nin > 1 && va && (ra & (P.part_py - 1)) == 0;
@@ -332,15 +342,15 @@ __device__ __forceinline__ void load_rhs(const SolveParams<T>& P, const T* const
         T a[8], b[8];
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-            a[r] = va && ok(r) ? __ldg(ia[0] + oa + col(r)) : T(0);
-            b[r] = vb && ok(r) ? __ldg(ib[0] + ob + col(r)) : T(0);
+            a[r] = ok(r) ? __ldg(ia[0] + oa + col(r)) : T(0);
+            b[r] = ok(r) ? __ldg(ib[0] + ob + col(r)) : T(0);
         }
         if (cx) {
             T c[8], d[8];
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
-                c[r] = va && ok(r) ? __ldg(ia[1] + oa + col(r)) : T(0);
-                d[r] = vb && ok(r) ? __ldg(ib[1] + ob + col(r)) : T(0);
+                c[r] = ok(r) ? __ldg(ia[1] + oa + col(r)) : T(0);
+                d[r] = ok(r) ? __ldg(ib[1] + ob + col(r)) : T(0);
             }
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
@@ -438,21 +448,18 @@ __device__ __forceinline__ void stream_item(const SolveParams<T>& P, int npairs,
     if constexpr (PH == 2) {
         // row s of the inverse x pass: modes s + 16 k, k = j + H r; k >= G/2
         // are the negated modes 16 - s + 16 (G - 1 - k)
-        const CT<T>* src = wk + (vp ? (size_t)pair * P.ld : 0);
+        // (a pair or row that does not exist reads one that does)
+        const int pe = vp ? pair : 0, se = act ? s : 0;
+        const CT<T>* lo = wk + (size_t)pe * P.ld + se * (G / 2) + j;
+        const CT<T>* hi = wk + (size_t)pe * P.ld + (se == 0 ? G : (16 - se) * (G / 2) + G - 1) - j;
+        const bool wall = se == 0 && j == 0;      // modes 0 and mx: r = 0 and 8
 #pragma unroll
         for (int r = 0; r < 16; ++r) {
-            const int k = j + H * r;
-            int pos, zero;
-            if (r < 8) {
-                pos = s * (G / 2) + k;
-                zero = s == 0 && k == 0;
-            } else {
-                pos = s == 0 ? G - k : (16 - s) * (G / 2) + G - 1 - k;
-                zero = s == 0 && k == G / 2;
-            }
             CT<T> x;
             x.x = x.y = T(0);
-            if (vp && !zero && QG_IN((long long)pair * P.ld + pos, nwk, 64)) x = src[pos];
+            if (!((r & 7) == 0 && wall) &&
+                QG_IN((r < 8 ? lo + H * r : hi - H * r) - wk, nwk, 64))
+                x = r < 8 ? lo[H * r] : hi[-H * r];
             v[r] = r < 8 ? Cplx<T>{x.x, x.y} : Cplx<T>{-x.x, -x.y};
         }
         row_fwd<T, LG>(v, row, j, tab);
@@ -474,8 +481,8 @@ __device__ __forceinline__ void stream_item(const SolveParams<T>& P, int npairs,
                     const int n = r < 8 ? tt + G * r : (16 - r) * G - tt;
                     CT<T> x;
                     x.x = x.y = T(0);
-                    if (vp && (tt > 0 || (r & 7) != 0) &&
-                        QG_IN((long long)pair * P.ld_tr + n - 1, ntr, 65))
+                    if ((tt > 0 || (r & 7) != 0) &&
+                        QG_IN((long long)(vp ? pair : 0) * P.ld_tr + n - 1, ntr, 65))
                         x = src[n];
                     v[r] = r < 8 ? Cplx<T>{x.x, x.y} : Cplx<T>{-x.x, -x.y};
                 }
@@ -490,34 +497,38 @@ __device__ __forceinline__ void stream_item(const SolveParams<T>& P, int npairs,
 
     if constexpr (PH == 1) {
         // mode-space solve of the modes l = s + 16 k, their images included
-        // (the eigenvalues of l and 2 my - l are the same); the walls l = 0
-        // and my stay 0
+        // (the eigenvalues of l and 2 my - l are the same)
         auto mode = [&](int pos) { return pos / (P.mx / 16) + 16 * (pos % (P.mx / 16)); };
         const int ka = OPY == 2 ? mode(pair) : mode(2 * pair);
         const int kb = OPY == 2 ? ka : mode(2 * pair + 1);
         const bool ok = vp && QG_IN(ka, P.mx + 1, 66) && QG_IN(kb, P.mx + 1, 66);
-        const T lxa = ok ? __ldg(P.lamx + ka) : T(1), lxb = ok ? __ldg(P.lamx + kb) : T(1);
-        const T* ly_s = P.lamyr + s * G;
+        // lamyr comes divided by P.scale, a power of two: so do lamx and Ro, and
+        // the scaling takes no operation per mode
+        const T inv = T(1) / P.scale;
+        const T lxa = (ok ? __ldg(P.lamx + ka) : T(1)) * inv, lxb = (ok ? __ldg(P.lamx + kb) : T(1)) * inv;
+        const T ro = P.Ro * P.scale;
+        const T* ly_s = P.lamyr + (act ? s : 0) * G;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const int k = row_k<LG>(j, i);
-            const bool wall = s == 0 && (k == 0 || k == G / 2);
-            const bool in = act && !wall && QG_IN(s * G + k, 9 * G, 67);
-            const T ly = in ? __ldg(ly_s + k) : T(1);
+            const T ly = QG_IN((act ? s : 0) * G + k, 9 * G, 67) ? __ldg(ly_s + k) : T(1);
             // the pair's 2 F are -Im Z and Re Z
             const T Fa = -v[i].y, Fb = v[i].x;
             T x, y;
             if (OPY == 1) {
-                x = Fa * (P.scale * recip(lxa + ly));
-                y = Fb * (P.scale * recip(lxb + ly));
+                x = Fa * recip(lxa + ly);
+                y = Fb * recip(lxb + ly);
             } else {
                 const T q1 = P.scale * Fa, q2 = P.scale * Fb;
-                const T al = P.Ro * (lxa + ly);
+                const T al = ro * (lxa + ly);
                 const T den = al * (al - P.f1 - P.f2);
                 x = (al * q1 - P.f2 * q1 - P.f1 * q2) / den;
                 y = (al * q2 - P.f2 * q1 - P.f1 * q2) / den;
             }
-            v[i] = in ? Cplx<T>{x, y} : Cplx<T>{T(0), T(0)};
+            v[i] = Cplx<T>{x, y};
+            // the walls l = 0 and my stay 0
+            if ((row_k0<LG>(i) == 0 || row_k0<LG>(i) == G / 2) && s == 0 && j == 0)
+                v[i] = Cplx<T>{T(0), T(0)};
         }
         row_bwd<T, LG>(v, row, j, tab);
         row_sync<LG>();
@@ -538,20 +549,29 @@ __device__ __forceinline__ void stream_item(const SolveParams<T>& P, int npairs,
             const bool vb = vp && rb <= P.my - 1;
             const long long nw = (long long)(P.my + 1) * P.ld;
             (void)nw;
-            T* oa = P.out[0] + (vp ? (size_t)ra * P.ld : 0);
-            T* ob = P.out[OPY == 2 ? 1 : 0] + (vp ? (size_t)rb * P.ld : 0);
-            // (column 0 and the wall row my are zero: out may be the array
-            // that held the scratch values)
+            T* oa = P.out[0] + (size_t)ra * P.ld;
+            T* ob = P.out[OPY == 2 ? 1 : 0] + (size_t)rb * P.ld;
+            // (columns 0 and mx and the wall row my are zero: out may be the
+            // array that held the scratch values.  Threads 0 and G/2 hold
+            // some columns twice, at r < 8 and r >= 8, and write them twice.)
+            if (vp) {
 #pragma unroll
-            for (int r = 0; r < 16; ++r) {
-                const bool second = r >= 8;
-                const int n = second ? (16 - r) * G - tt : tt + G * r;
-                const bool wall = tt == 0 && (r & 7) == 0;      // n = 0 or N
-                if (second && !wall && (tt == 0 || tt == G / 2)) continue;   // seen at r < 8
-                const T sg = second ? T(-1) : T(1);
-                const T fa = wall ? T(0) : -sg * v[r].y, fb = wall || !vb ? T(0) : sg * v[r].x;
-                if (vp && QG_IN((long long)ra * P.ld + n, nw, 70)) oa[n] = fa;
-                if (vp && QG_IN((long long)rb * P.ld + n, nw, 70)) ob[n] = fb;
+                for (int r = 0; r < 16; ++r) {
+                    const bool second = r >= 8;
+                    const int n = second ? (16 - r) * G - tt : tt + G * r;
+                    const T sg = second ? T(-1) : T(1);
+                    T fa = -sg * v[r].y, fb = sg * v[r].x;
+                    if ((r & 7) == 0 && tt == 0) fa = fb = T(0);
+                    if (QG_IN((long long)ra * P.ld + n, nw, 70)) oa[n] = fa;
+                    if (QG_IN((long long)rb * P.ld + n, nw, 70)) ob[n] = fb;
+                }
+                if (!vb) {
+#pragma unroll
+                    for (int r = 0; r < 16; ++r) {
+                        const int n = r >= 8 ? (16 - r) * G - tt : tt + G * r;
+                        if (QG_IN((long long)rb * P.ld + n, nw, 70)) ob[n] = T(0);
+                    }
+                }
             }
         }
     } else {
@@ -570,7 +590,7 @@ __device__ __forceinline__ void stream_item(const SolveParams<T>& P, int npairs,
                     const int pos = low ? s * (G / 2) + k : (16 - s) * (G / 2) + G - 1 - k;
                     const T sg = low ? T(1) : T(-1);
                     Cplx<T> o{-sg * v[i].y, sg * v[i].x};
-                    if (pos == 0) o = Cplx<T>{T(0), T(0)};      // the wall mode
+                    if (i == 0 && s == 0 && j == 0) o = Cplx<T>{T(0), T(0)};   // the wall mode
                     sts_<T>(stg, pos * SP + grp, o, SLIM);
                 }
             }
@@ -580,8 +600,9 @@ __device__ __forceinline__ void stream_item(const SolveParams<T>& P, int npairs,
                 for (int r = 0; r < 16; ++r) {
                     const bool second = r >= 8;
                     const int n = second ? (16 - r) * G - tt : tt + G * r;
-                    if (tt == 0 && (r & 7) == 0) continue;
-                    if (second && (tt == 0 || tt == G / 2)) continue;
+                    // (elements 0 and N are walls: N has no place; threads 0 and
+                    // G/2 hold some elements twice)
+                    if (r == 8 && tt == 0) continue;
                     const T sg = second ? T(-1) : T(1);
                     sts_<T>(stg, n * SP + grp, Cplx<T>{-sg * v[r].y, sg * v[r].x}, SLIM);
                 }
