@@ -1162,6 +1162,20 @@ qg_status stage_fused(qg_ctx* h, int s_idx, cudaStream_t s) {
     return QG_OK;
 }
 
+template <typename T>
+InitPartials<T> init_params(qg_ctx* h, const LevelTables& t, int L) {
+    InitPartials<T> q;
+    q.w = plane<T>(h->w[0], h->plane_f, L);
+    q.part = plane<T>(h->part, h->plane_c, 4 * L);
+    q.plane = h->plane_c;
+    q.ldf = h->ldf;
+    q.ldc = t.ldc;
+    q.mx = t.mx;
+    q.my = t.my;
+    q.levels = h->levels;
+    return q;
+}
+
 // Restriction of the current state into the partial planes (plane 0 holds
 // the complete values, planes 1-3 zero), needed once after qg_set_state.
 template <typename T>
@@ -1169,11 +1183,8 @@ qg_status init_partials(qg_ctx* h, cudaStream_t s) {
     const LevelTables* t = nullptr;
     qg_status st = get_level(h, h->levels, &t);
     if (st != QG_OK) return fail(h, st);
-    QG_TRY(cudaMemsetAsync(h->part, 0, 4 * (size_t)h->layers * h->plane_c * sizeof(T), s));
     for (int L = 0; L < h->layers; ++L)
-        QG_TRY(launch_restrict<T>(plane<T>(h->w[0], h->plane_f, L), h->ldf,
-                                  plane<T>(h->part, h->plane_c, 4 * L), t->ldc, t->mx, t->my,
-                                  h->levels, s));
+        QG_TRY(launch_init_partials<T>(init_params<T>(h, *t, L), nullptr, 1, s));
     return QG_OK;
 }
 
@@ -1489,17 +1500,17 @@ qg_status qg_set_state(qg_handle h, const void* field, int layer) {
         QG_TRY(cudaMemcpyAsync(h->stage_in[b], field, bytes, cudaMemcpyHostToDevice, h->xin));
         QG_TRY(cudaEventRecord(h->in_ready[b], h->xin));
         QG_TRY(cudaStreamWaitEvent(h->stream, h->in_ready[b], 0));
-        QG_TRY(copy_in(dst, h->ldf, h->stage_in[b], h->nx - 1, h->ny - 1, h->esz, h->stream));
+        QG_TRY(copy_in(dst, h->ldf, h->stage_in[b], h->nx - 1, h->ny - 1, h->esz, h->stream,
+                       h->dclock));
         QG_TRY(cudaEventRecord(h->in_free[b], h->stream));
     } else {
-        QG_TRY(copy_in(dst, h->ldf, field, h->nx - 1, h->ny - 1, h->esz, h->stream));
+        QG_TRY(copy_in(dst, h->ldf, field, h->nx - 1, h->ny - 1, h->esz, h->stream, h->dclock));
     }
     h->part_valid = false;
     h->time_host = 0.0;
     if (h->solver == QG_SOLVER_MULTIGRID)   // the first solve's guess: zero
         QG_TRY(cudaMemsetAsync(h->levels ? h->cpsi : h->psi, 0,
                                (h->levels ? h->plane_c : h->plane_f) * h->esz, h->stream));
-    QG_TRY(cudaMemsetAsync(h->dclock, 0, sizeof(double) * 4, h->stream));
     return QG_OK;
 }
 
@@ -2401,6 +2412,7 @@ struct qg_ensemble_s {
     std::vector<uint64_t> gen;              // members' graph_gen when it was captured
     std::vector<EnsSolveGroup> sg;
     std::vector<void*> dallocs;             // device tables of the batched launches
+    void* dinit = nullptr;                  // InitPartials of the coarsened members
     int64_t kernels = 0;
     bool fresh = false;                     // members hold no user state yet
 };
@@ -2410,6 +2422,7 @@ namespace {
 void ensemble_tables_free(qg_ensemble e) {
     for (void* p : e->dallocs) cudaFree(p);
     e->dallocs.clear();
+    e->dinit = nullptr;
     e->sg.clear();
 }
 
@@ -2632,6 +2645,20 @@ qg_status ensemble_tables(qg_ensemble e) {
                            cudaMemcpyHostToDevice) != cudaSuccess)
                 return QG_ERR_CUDA;
         }
+    }
+    std::vector<InitPartials<T>> ini;
+    for (qg_ctx* h : e->m) {
+        if (!h->part) continue;
+        const LevelTables* t = nullptr;
+        qg_status st = get_level(h, h->levels, &t);
+        if (st != QG_OK) return st;
+        ini.push_back(init_params<T>(h, *t, 0));
+    }
+    if (!ini.empty()) {
+        QG_TRY_E(ens_alloc(e, &e->dinit, ini.size() * sizeof(ini[0])));
+        if (cudaMemcpy(e->dinit, ini.data(), ini.size() * sizeof(ini[0]), cudaMemcpyHostToDevice) !=
+            cudaSuccess)
+            return QG_ERR_CUDA;
     }
     // each group's solve engine, timed over whole group steps on the
     // members' buffers (which then return to rest) while the members hold
@@ -2950,17 +2977,34 @@ qg_status qg_ensemble_step(qg_ensemble e, int64_t n) {
     for (qg_ctx* h : e->m)
         if (h->latched != QG_OK) return qg_last_error(h);
     if (n == 0) return QG_OK;
-    // the members' partial sums of R^l w^n are made on the ensemble stream
+    // the members' partial sums of R^l w^n are made on the ensemble stream: in
+    // one launch when every coarsened member needs them
+    qg_status s = ensemble_build(e);
+    if (s != QG_OK) return s;
+    int with = 0, stale = 0;
+    for (qg_ctx* h : e->m)
+        if (h->part) {
+            ++with;
+            stale += !h->part_valid;
+        }
+    if (stale > 1 && stale == with && e->dinit) {
+        const bool f64 = e->m[0]->dtype == QG_F64;
+        const cudaError_t ei =
+            f64 ? launch_init_partials<double>({}, static_cast<const InitPartials<double>*>(e->dinit),
+                                               with, e->stream)
+                : launch_init_partials<float>({}, static_cast<const InitPartials<float>*>(e->dinit),
+                                              with, e->stream);
+        if (ei != cudaSuccess) return QG_ERR_CUDA;
+        for (qg_ctx* h : e->m) h->part_valid = h->part != nullptr;
+    }
     for (qg_ctx* h : e->m) {
         if (h->part && !h->part_valid) {
-            const qg_status s = h->dtype == QG_F64 ? init_partials<double>(h, h->stream)
-                                                   : init_partials<float>(h, h->stream);
+            s = h->dtype == QG_F64 ? init_partials<double>(h, h->stream)
+                                   : init_partials<float>(h, h->stream);
             if (s != QG_OK) return s;
             h->part_valid = true;
         }
     }
-    qg_status s = ensemble_build(e);
-    if (s != QG_OK) return s;
     for (qg_ctx* h : e->m)
         if (h->stats) h->stat_count += n;
     for (int64_t k = 0; k < n; ++k)

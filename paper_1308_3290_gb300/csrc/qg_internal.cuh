@@ -160,6 +160,19 @@ template <typename T>
 cudaError_t launch_prolong(const T* coarse, int ldc, T* fine, int ldf,
                            int nx, int ny, int levels, cudaStream_t s);
 
+// R^l w into the four partial planes of a step (stencil.cu): of one basin, or
+// (table non-null, n entries in device memory) of every member of an ensemble.
+template <typename T>
+struct InitPartials {
+    const T* w;
+    T* part;
+    size_t plane;                // elements between the planes
+    int ldf, ldc, mx, my, levels;
+};
+template <typename T>
+cudaError_t launch_init_partials(const InitPartials<T>& one, const InitPartials<T>* table, int n,
+                                 cudaStream_t s);
+
 // The same on fields in the exchange layout (device memory, not overlapping).
 template <typename T>
 cudaError_t launch_restrict_dense(const T* fine, T* coarse, int nx, int ny, int levels,
@@ -418,8 +431,9 @@ int bounds_site_dense();
 // Whether ptr is device memory (not host or managed).
 bool on_device(const void* ptr);
 // Copies between the dense exchange layout and the padded node layout.
+// (clear: four doubles to set to zero in the same launch, or null)
 cudaError_t copy_in(void* padded, int ld, const void* dense, int nxm1,
-                    int nym1, size_t esz, cudaStream_t s);
+                    int nym1, size_t esz, cudaStream_t s, double* clear = nullptr);
 cudaError_t copy_out(void* dense, const void* padded, int ld, int nxm1,
                      int nym1, size_t esz, cudaStream_t s);
 

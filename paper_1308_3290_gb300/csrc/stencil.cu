@@ -60,12 +60,8 @@ __global__ void fine_stage2_kernel(const T* __restrict__ psi1,
 // R^l as one hat-weighted sum: with f = 2^l, the composed full weighting has
 // separable weights (f - |d|)/f^2 per direction for |d| < f.
 template <typename T>
-__global__ void restrict_kernel(const T* __restrict__ fine, int ldf,
-                                T* __restrict__ coarse, int ldc, int mx,
-                                int my, int levels) {
-    const int I = blockIdx.x * blockDim.x + threadIdx.x + 1;
-    const int J = blockIdx.y * blockDim.y + threadIdx.y + 1;
-    if (I >= mx || J >= my) return;
+__device__ __forceinline__ T restricted_at(const T* __restrict__ fine, int ldf, int I, int J, int my,
+                                           int levels) {
     const int f = 1 << levels;
     const T* base = fine + (size_t)(f * J) * ldf + f * I;
     // the fine grid has (f my + 1) rows of pitch ldf
@@ -81,8 +77,37 @@ __global__ void restrict_kernel(const T* __restrict__ fine, int ldf,
         acc += T(f - (dj < 0 ? -dj : dj)) * racc;
     }
     const T inv = T(1) / (T(f) * T(f) * T(f) * T(f));
+    return acc * inv;
+}
+
+template <typename T>
+__global__ void restrict_kernel(const T* __restrict__ fine, int ldf,
+                                T* __restrict__ coarse, int ldc, int mx,
+                                int my, int levels) {
+    const int I = blockIdx.x * blockDim.x + threadIdx.x + 1;
+    const int J = blockIdx.y * blockDim.y + threadIdx.y + 1;
+    if (I >= mx || J >= my) return;
     if (QG_IN((long long)J * ldc + I, (long long)(my + 1) * ldc, 42))
-        coarse[(size_t)J * ldc + I] = acc * inv;
+        coarse[(size_t)J * ldc + I] = restricted_at(fine, ldf, I, J, my, levels);
+}
+
+// R^l w into a step's partial planes: plane 0 whole, planes 1 to 3 zero.
+// Launch-bound: member blockIdx.y of an ensemble takes its arrays from the
+// table, so that one launch serves all members (a memset and a restriction
+// each took 460 us for 48 basins, the batched launch some 40 with its wait).
+template <typename T>
+__global__ void __launch_bounds__(256) init_partials_kernel(InitPartials<T> one,
+                                                            const InitPartials<T>* table) {
+    const InitPartials<T> q = table ? table[blockIdx.y] : one;
+    const int n = q.mx * q.my, lx = 31 - __clz(q.mx);   // (sides are powers of two)
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+        const int I = e & (q.mx - 1), J = e >> lx;
+        if (I < 1 || J < 1) continue;
+        const size_t o = (size_t)J * q.ldc + I;
+        if (!QG_IN((long long)o, (long long)(q.my + 1) * q.ldc, 42)) continue;
+        q.part[o] = restricted_at(q.w, q.ldf, I, J, q.my, q.levels);
+        for (int k = 1; k < 4; ++k) q.part[k * q.plane + o] = T(0);
+    }
 }
 
 // P^l as bilinear interpolation from the coarse nodes around each fine node.
@@ -133,6 +158,18 @@ cudaError_t launch_restrict(const T* fine, int ldf, T* coarse, int ldc, int mx,
     const dim3 block(32, 8);
     const dim3 grid((mx - 1 + 31) / 32, (my - 1 + 7) / 8);
     restrict_kernel<T><<<grid, block, 0, s>>>(fine, ldf, coarse, ldc, mx, my, levels);
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_init_partials(const InitPartials<T>& one, const InitPartials<T>* table, int n,
+                                 cudaStream_t s) {
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    long blocks = table ? 2L * nsm : ((long)one.mx * one.my + 255) / 256;
+    if (blocks > 8L * nsm) blocks = 8L * nsm;
+    init_partials_kernel<T><<<dim3((unsigned)blocks, table ? n : 1), 256, 0, s>>>(one, table);
     return cudaGetLastError();
 }
 
@@ -427,7 +464,9 @@ cudaError_t launch_mean_out(T* dense, const double* acc, int ldacc, double scale
 // per element the index arithmetic was the kernel's time).
 template <typename W, bool TO_PADDED>
 __global__ void __launch_bounds__(256)
-repack_kernel(W* __restrict__ dst, const W* __restrict__ src, unsigned nxm1, unsigned nym1, int ld) {
+repack_kernel(W* __restrict__ dst, const W* __restrict__ src, unsigned nxm1, unsigned nym1, int ld,
+              double* clear) {
+    if (clear && blockIdx.x == 0 && threadIdx.x < 4) clear[threadIdx.x] = 0.0;
     constexpr unsigned V = 16 / sizeof(W);
     const unsigned n = nxm1 * nym1, stride = gridDim.x * blockDim.x;
     const unsigned t0 = blockIdx.x * blockDim.x + threadIdx.x;
@@ -480,7 +519,7 @@ static const void* device_view(const void* ptr) {
 }
 
 static cudaError_t repack(void* dst, const void* src, int nxm1, int nym1, int ld, size_t esz,
-                          bool to_padded, cudaStream_t s) {
+                          bool to_padded, cudaStream_t s, double* clear = nullptr) {
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -491,10 +530,10 @@ static cudaError_t repack(void* dst, const void* src, int nxm1, int nym1, int ld
         using W = decltype(w);
         if (to_padded)
             repack_kernel<W, true><<<(int)blocks, 256, 0, s>>>(static_cast<W*>(dst),
-                                                               static_cast<const W*>(src), nxm1, nym1, ld);
+                                                               static_cast<const W*>(src), nxm1, nym1, ld, clear);
         else
             repack_kernel<W, false><<<(int)blocks, 256, 0, s>>>(static_cast<W*>(dst),
-                                                                static_cast<const W*>(src), nxm1, nym1, ld);
+                                                                static_cast<const W*>(src), nxm1, nym1, ld, clear);
     };
     if (esz == 8) go(double());
     else go(float());
@@ -514,8 +553,13 @@ bool on_device(const void* ptr) {
 // C2C link, which beats a DMA copy plus a device repack) are repacked by a
 // kernel; pageable host buffers go through 2-D copies.
 cudaError_t copy_in(void* padded, int ld, const void* dense, int nxm1, int nym1,
-                    size_t esz, cudaStream_t s) {
-    if (const void* v = device_view(dense)) return repack(padded, v, nxm1, nym1, ld, esz, true, s);
+                    size_t esz, cudaStream_t s, double* clear) {
+    if (const void* v = device_view(dense))
+        return repack(padded, v, nxm1, nym1, ld, esz, true, s, clear);
+    if (clear) {
+        const cudaError_t e = cudaMemsetAsync(clear, 0, 4 * sizeof(double), s);
+        if (e != cudaSuccess) return e;
+    }
     char* dst = static_cast<char*>(padded) + (size_t)(ld + 1) * esz;
     return cudaMemcpy2DAsync(dst, (size_t)ld * esz, dense, (size_t)nxm1 * esz,
                              (size_t)nxm1 * esz, nym1, cudaMemcpyDefault, s);
@@ -540,6 +584,8 @@ cudaError_t copy_out(void* dense, const void* padded, int ld, int nxm1, int nym1
                                             cudaStream_t);                          \
     template cudaError_t launch_prolong<T>(const T*, int, T*, int, int, int, int,   \
                                            cudaStream_t);                            \
+    template cudaError_t launch_init_partials<T>(const InitPartials<T>&, const InitPartials<T>*, \
+                                                 int, cudaStream_t);                \
     template cudaError_t launch_restrict_dense<T>(const T*, T*, int, int, int, cudaStream_t); \
     template cudaError_t launch_prolong_dense<T>(const T*, T*, int, int, int, cudaStream_t); \
     template cudaError_t launch_cfl_max<T>(const T*, int, int, int, int, double,     \
