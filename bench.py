@@ -161,7 +161,7 @@ def measured_peaks():
 # the source files each kernel class is built from
 KERNEL_SOURCES = {
     "fine": ["fused.cu", "qg_internal.cuh"],
-    "solve": ["solve32.cu", "solve.cu", "dst_engine.cuh", "qg_internal.cuh"],
+    "solve": ["solve_stream.cu", "solve32.cu", "dst_engine.cuh", "qg_internal.cuh"],
 }
 
 

@@ -647,7 +647,8 @@ qg_status solve_level(qg_ctx* h, const LevelTables& t, const void* in, void* tr,
 // values per thread, engines 32, 33, 34; or, on small one-layer FP32 grids,
 // the matrix-form solve on the tensor cores of solve_mtx.cu, engine 40, or
 // the same with tcgen05 and TMEM accumulators, engine 41 (solve_tc.cu); or
-// the half-length sine transforms of solve_stream.cu, engine 50) is
+// the half-length sine transforms of solve_stream.cu, engine 50; or, up to
+// 256 intervals a side, the sine sums of solve_dense.cu, engine 42) is
 // chosen per handle when it is created, by timing a few whole steps with each
 // engine that supports the elliptic grid (the solve alone, timed back to
 // back, ranks them differently: in a step the fine sweep has just streamed

@@ -283,8 +283,9 @@ def qg_set_solver(h: int, kind: int, cycles: int = 4) -> None:
 
 def qg_solve_engine(h: int) -> int:
     """The elliptic-solve kernel of the handle's step: 4, 16 (shared-memory
-    FFT), 32, 33, 34 (warp-group FFT), 40 (matrix form on the tensor cores),
-    0 (multigrid)."""
+    FFT), 32, 33, 34 (warp-group FFT), 40 and 41 (matrix form on the tensor
+    cores), 42 (sine sums, one output per thread), 50 (half-length sine
+    transforms), 0 (multigrid)."""
     e = ctypes.c_int32()
     _check(load().qg_solve_engine(h, ctypes.byref(e)), "qg_solve_engine")
     return e.value
