@@ -521,9 +521,13 @@ __device__ __forceinline__ void stream_item(const SolveParams<T>& P, int npairs,
             } else {
                 const T q1 = P.scale * Fa, q2 = P.scale * Fb;
                 const T al = ro * (lxa + ly);
-                const T den = al * (al - P.f1 - P.f2);
-                x = (al * q1 - P.f2 * q1 - P.f1 * q2) / den;
-                y = (al * q2 - P.f2 * q1 - P.f1 * q2) / den;
+                // (the determinant al (al - f1 - f2) factor by factor, both
+                // negative: no underflow, and no division, whose rare path
+                // splits the chains of the 16 modes: FP32 256 x 256, l = 0,
+                // 51.4 us a step with two divisions a mode, 43.1 with one)
+                const T r = recip(al) * recip(al - P.f1 - P.f2);
+                x = (al * q1 - P.f2 * q1 - P.f1 * q2) * r;
+                y = (al * q2 - P.f2 * q1 - P.f1 * q2) * r;
             }
             v[i] = Cplx<T>{x, y};
             // the walls l = 0 and my stay 0
@@ -823,20 +827,29 @@ cudaError_t launch_ppc(const SolveParams<T>& P, int npairs, cudaStream_t s) {
 // 512 x 2048 64.4 with (4, 1, 4), 69.8 with (8, 1, 4); 2048 x 4096 291 with
 // (2, 1, 2), 298 with (4, 1, 1); FP64 512 x 1024 575 with (4, 2, 4), 661
 // with (4, 2, 1).
+// Two layers in FP32 store one value of each layer per pair and element, 8
+// bytes: the two passes that write the scratch arrays take four pairs at
+// least, a 32-byte sector (l = 0, 1024 x 2048: 182 us with (4, 4, 2), 222 with
+// (1, 1, 1), 197 with (2, 2, 1); 256 x 256 36.9, 39.0 and 39.0).
 template <typename T>
 __host__ __device__ constexpr int ppc_max(int lg) {
     return lg <= 10 ? 8 : lg == 11 ? 4 : lg == 12 ? (sizeof(T) == 4 ? 4 : 2) : 1;
 }
+template <typename T, int OPY, int PH>
+__host__ __device__ constexpr int ppc_min(int lg) {
+    const int least = OPY == 2 && PH < 2 && sizeof(T) == 4 ? 4 : 1;
+    return least < ppc_max<T>(lg) ? least : ppc_max<T>(lg);
+}
 template <typename T>
-int pick_ppc(int ph, int lg, int npairs, int batch, int nsm) {
+int pick_ppc(int ph, int lg, int npairs, int batch, int nsm, int least) {
     const int tp = 9 * (1 << lg) / 256;
-    int best = 1, cost = 0;
-    for (int c = 1; c <= ppc_max<T>(lg); c *= 2) {
+    int best = least, cost = 0;
+    for (int c = least; c <= ppc_max<T>(lg); c *= 2) {
         const int ctas = (npairs + c - 1) / c * batch;
         const int w = (ctas + nsm - 1) / nsm * (round32(tp * c) / 32);
         const bool keep_tie = ph == 2 && sizeof(T) == 4;
-        if (c == 1 || w < cost || (w == cost && !keep_tie)) {
-            if (c > 1 && cost <= 16 && 8 * cost <= 9 * w) continue;
+        if (c == least || w < cost || (w == cost && !keep_tie)) {
+            if (c > least && cost <= 16 && 8 * cost <= 9 * w) continue;
             best = c;
             cost = w;
         }
@@ -849,18 +862,21 @@ cudaError_t launch_pass(const SolveParams<T>& P, int npairs, cudaStream_t s) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const int c = pick_ppc<T>(PH, LG, npairs, P.batch ? P.nbatch : 1, nsm);
-    constexpr int M = ppc_max<T>(LG);
+    constexpr int M = ppc_max<T>(LG), LEAST = ppc_min<T, OPY, PH>(LG);
+    const int c = pick_ppc<T>(PH, LG, npairs, P.batch ? P.nbatch : 1, nsm, LEAST);
     if constexpr (M >= 8) {
         if (c == 8) return launch_ppc<T, OPY, PH, LG, 8>(P, npairs, s);
     }
     if constexpr (M >= 4) {
         if (c == 4) return launch_ppc<T, OPY, PH, LG, 4>(P, npairs, s);
     }
-    if constexpr (M >= 2) {
+    if constexpr (M >= 2 && LEAST <= 2) {
         if (c == 2) return launch_ppc<T, OPY, PH, LG, 2>(P, npairs, s);
     }
-    return launch_ppc<T, OPY, PH, LG, 1>(P, npairs, s);
+    if constexpr (LEAST == 1) {
+        return launch_ppc<T, OPY, PH, LG, 1>(P, npairs, s);
+    }
+    return cudaErrorInvalidValue;   // (not reached: c is one of the above)
 }
 
 template <typename T, int OPY, int PH>
