@@ -277,8 +277,9 @@ qg_status qg_set_solver(qg_handle h, qg_solver kind, int32_t cycles);
  * pointer): chosen when the handle is created by timing whole steps with
  * every candidate that supports the elliptic grid (the QG_SOLVE_ENGINE
  * environment variable forces a supported one; the choice and the stencil
- * tile are cached per grid for the process and, when QG_TUNE_CACHE names a
- * file, in that file).  4 or 16: shared-memory
+ * tile are cached per grid, for basins and for ensemble members apart, for the
+ * process and, when QG_TUNE_CACHE names a file, in that file; a choice made
+ * with the engine or the tile forced is not).  4 or 16: shared-memory
  * Stockham FFT with base radix 4 or 16; 32, 33, 34: warp-group FFT with 32,
  * 16 or 8 values per thread; 40: the sine sums as dense matrix products on
  * the tensor cores, 3xTF32 (FP32 grids of at most 64 x 128 or 128 x 64

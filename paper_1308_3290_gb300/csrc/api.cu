@@ -653,10 +653,11 @@ qg_status solve_level(qg_ctx* h, const LevelTables& t, const void* in, void* tr,
 // engine that supports the elliptic grid (the solve alone, timed back to
 // back, ranks them differently: in a step the fine sweep has just streamed
 // its fields through L2), and the fastest is kept.  Results are cached per
-// (nx, ny, levels, layers, dtype) for the process and, when the environment
+// (nx, ny, levels, layers, dtype, member) for the process and, when the environment
 // variable QG_TUNE_CACHE names a file, in that file (one line
-// "nx ny levels layers esz engine rows ry" per entry; ensemble groups add
-// lines "group mx my dx dy members esz engine").  QG_SOLVE_ENGINE=4|16|32|33|34|40|41|42|50
+// "nx ny levels layers esz engine rows ry" per entry, for an ensemble member
+// with "member" before it; ensemble groups add lines "group mx my dx dy
+// members esz engine").  QG_SOLVE_ENGINE=4|16|32|33|34|40|41|42|50
 // forces a choice where that engine supports the grid.  Other grids use the
 // size rule.
 
@@ -707,7 +708,9 @@ qg_status fine_maps(qg_ctx* h) {
     return QG_OK;
 }
 
-using TuneKey = std::tuple<int, int, int, int, int>;
+// (nx, ny, levels, layers, element size, ensemble member): a member's
+// candidates are others than a basin's (one tile, no sine sums)
+using TuneKey = std::tuple<int, int, int, int, int, int>;
 std::mutex g_tune_mutex;
 struct TuneVal {
     int engine, rows, ry;   // solve engine; fine rows per CTA and per thread
@@ -741,10 +744,12 @@ void tune_file_load() {
                 std::lock_guard<std::mutex> lock(g_batch_tune_mutex);
                 g_batch_tune[GroupKey(a, b, dx, dy, c, x)] = e;
             }
-        } else if (std::sscanf(line, "%d %d %d %d %d %d %d %d", &a, &b, &c, &d, &x, &e, &r, &y) == 8 &&
-                   known_engine(e) && fine_rows_supported((size_t)x, d, c, r, y)) {
-            g_tune_cache[TuneKey(a, b, c, d, x)] = {e, r, y};
+            continue;
         }
+        const int m = std::strncmp(line, "member ", 7) == 0 ? 1 : 0;
+        if (std::sscanf(line + 7 * m, "%d %d %d %d %d %d %d %d", &a, &b, &c, &d, &x, &e, &r, &y) == 8 &&
+            known_engine(e) && fine_rows_supported((size_t)x, d, c, r, y))
+            g_tune_cache[TuneKey(a, b, c, d, x, m)] = {e, r, y};
     }
     std::fclose(f);
 }
@@ -754,8 +759,9 @@ void tune_file_store(const TuneKey& k, const TuneVal& v) {
     if (!path) return;
     FILE* f = std::fopen(path, "a");
     if (!f) return;
-    std::fprintf(f, "%d %d %d %d %d %d %d %d\n", std::get<0>(k), std::get<1>(k), std::get<2>(k),
-                 std::get<3>(k), std::get<4>(k), v.engine, v.rows, v.ry);
+    std::fprintf(f, "%s%d %d %d %d %d %d %d %d\n", std::get<5>(k) ? "member " : "", std::get<0>(k),
+                 std::get<1>(k), std::get<2>(k), std::get<3>(k), std::get<4>(k), v.engine, v.rows,
+                 v.ry);
     std::fclose(f);
 }
 
@@ -866,7 +872,7 @@ qg_status autotune_solve(qg_ctx* h) {
             return QG_OK;
         }
     }
-    const TuneKey key(h->nx, h->ny, h->levels, h->layers, (int)h->esz);
+    const TuneKey key(h->nx, h->ny, h->levels, h->layers, (int)h->esz, h->member ? 1 : 0);
     {
         std::lock_guard<std::mutex> lock(g_tune_mutex);
         tune_file_load();
@@ -920,7 +926,8 @@ qg_status autotune_solve(qg_ctx* h) {
     }
     // the timing steps ran on the handle's buffers: return them to rest
     QG_TRY_S(rest_buffers(h, h->stream));
-    if (force) return QG_OK;   // (a choice among some of the engines is not kept)
+    // (a choice among some of the engines or tiles is not kept)
+    if (force || (forced_rows && tiles.size() > 1)) return QG_OK;
     std::lock_guard<std::mutex> lock(g_tune_mutex);
     const TuneVal v{h->solve_engine, h->fine_rows, h->fine_ry};
     g_tune_cache[key] = v;
