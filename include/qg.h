@@ -275,7 +275,8 @@ qg_status qg_set_solver(qg_handle h, qg_solver kind, int32_t cycles);
 
 /* qg_solve_engine -- which kernel the step's elliptic solves run on (host
  * pointer): chosen when the handle is created by timing whole steps with
- * every candidate that supports the elliptic grid (the QG_SOLVE_ENGINE
+ * the candidates that support the elliptic grid (where 50 or 42 takes it, 16,
+ * 32 and 41, in FP32 also 4 and 33, are not timed: they lose; the QG_SOLVE_ENGINE
  * environment variable forces a supported one; the choice and the stencil
  * tile are cached per grid, for basins and for ensemble members apart, for the
  * process and, when QG_TUNE_CACHE names a file, in that file; a choice made

@@ -73,3 +73,38 @@ print(json.dumps(choice(b.h)))
     assert not cache.exists() or cache.read_text() == ""
     got = run(body, cache)
     assert cache.read_text().split() == ["64", "128", "1", "1", "4"] + [str(v) for v in got]
+
+
+@pytest.mark.parametrize("dtype,esz", [("f64", 8), ("f32", 4)])
+def test_a_forced_engine_that_does_not_take_the_grid(tmp_path, dtype, esz):
+    """64 x 128, l = 1 is too short for engine 50: the choice is among the others
+    but the sine sums (42), with an empty cache and with one that names 42, and
+    is not kept."""
+    require_gpu()
+    cache = tmp_path / "tune.txt"
+    body = f"""
+b = qg.Basin(dtype="{dtype}", **kw)
+print(json.dumps(choice(b.h)))
+"""
+    line = f"64 128 1 1 {esz} 42 8 1\n"
+    for text in ("", line):
+        cache.write_text(text)
+        assert run(body, cache, QG_SOLVE_ENGINE="50")[0] not in (42, 50)
+        assert cache.read_text() == text
+
+
+@pytest.mark.parametrize("nx,ny,levels,dtype,never", [
+    (64, 128, 1, "f32", (4, 16, 32, 33, 41)), (64, 128, 1, "f64", (16, 32)),
+    (512, 1024, 0, "f32", (4, 16, 32, 33)), (512, 1024, 0, "f64", (16, 32))])
+def test_engines_that_are_not_timed(tmp_path, nx, ny, levels, dtype, never):
+    """Where engine 42 or 50 takes the grid, some engines are not candidates; on
+    a grid that neither takes (8 x 512) another one is found."""
+    require_gpu()
+    body = f"""
+b = qg.Basin({nx}, {ny}, Re=200.0, Ro=0.0016, levels={levels}, dt=1e-5, dtype="{dtype}")
+c = qg.Basin(8, 512, Re=200.0, Ro=0.0016, levels=0, dt=1e-5, dtype="{dtype}")
+print(json.dumps([qg.qg_solve_engine(b.h), qg.qg_solve_engine(c.h)]))
+"""
+    got = run(body, tmp_path / "tune.txt")
+    assert got[0] not in never
+    assert got[1] in (4, 16, 32, 33, 34)
