@@ -2020,28 +2020,23 @@ static qg_status diagnostics_sums(qg_ctx* h, const float* lo, cudaStream_t s) {
 }
 
 // After project: h->psi + *lo is the streamfunction of w^n refined once on
-// the elliptic grid (FP32, one layer, sine transforms).  *scratch holds lo;
-// the caller frees it.
-static qg_status refine_psi(qg_ctx* h, void** scratch, const float** lo) {
+// the elliptic grid (FP32, one layer, sine transforms).  In the handle's own
+// fields, so that nothing is allocated: the residual and its solution in cw
+// (its walls cleared: the solves read them as zeros), lo in w[1], which the
+// next step's first stage overwrites.
+static qg_status refine_psi(qg_ctx* h, const float** lo) {
     const LevelTables* t = nullptr;
     qg_status st = get_level(h, h->levels, &t);
     if (st != QG_OK) return fail(h, st);
-    const size_t pc = h->plane_c;
-    QG_TRY(scratch_alloc(h, scratch, (2 * pc + h->plane_f) * sizeof(float)));
-    float *r = static_cast<float*>(*scratch), *d = r + pc, *l = d + pc;
+    float *r = static_cast<float*>(h->cw), *l = static_cast<float*>(h->w[1]);
     float* psi = static_cast<float*>(h->levels ? h->cpsi : h->psi);
-    cudaError_t e = cudaMemsetAsync(d, 0, pc * sizeof(float), h->stream);
-    if (e == cudaSuccess)
-        e = launch_residual(static_cast<const float*>(h->w[0]), h->ldf, psi, r, t->ldc, t->mx, t->my,
-                            h->levels, 1.0 / (t->dxc * t->dxc), 1.0 / (t->dyc * t->dyc), h->stream);
-    if (e == cudaSuccess)
-        st = solve_level<float>(h, *t, r, h->ct, h->ld_t, h->plane_t, h->cw, d, pc, h->stream);
-    if (e == cudaSuccess && st == QG_OK)
-        e = launch_prolong_pair(psi, d, t->ldc, static_cast<float*>(h->psi), l, h->ldf, h->nx, h->ny,
-                                h->levels, h->stream);
-    if (e != cudaSuccess || st != QG_OK) cudaFreeAsync(*scratch, h->stream);
+    QG_TRY(cudaMemsetAsync(r, 0, h->plane_c * sizeof(float), h->stream));
+    QG_TRY(launch_residual(static_cast<const float*>(h->w[0]), h->ldf, psi, r, t->ldc, t->mx, t->my,
+                           h->levels, 1.0 / (t->dxc * t->dxc), 1.0 / (t->dyc * t->dyc), h->stream));
+    st = solve_level<float>(h, *t, r, h->ct, h->ld_t, h->plane_t, r, r, h->plane_c, h->stream);
     if (st != QG_OK) return st;
-    QG_TRY(e);
+    QG_TRY(launch_prolong_pair(psi, r, t->ldc, static_cast<float*>(h->psi), l, h->ldf, h->nx, h->ny,
+                               h->levels, h->stream));
     *lo = l;
     return QG_OK;
 }
@@ -2052,14 +2047,12 @@ qg_status qg_diagnostics(qg_handle h, double* ke, double* enstrophy, double* max
     if (h->latched != QG_OK) return qg_last_error(h);
     qg_status s = project_any(h, h->w[0], h->stream);
     if (s != QG_OK) return s;
-    void* scratch = nullptr;
     const float* lo = nullptr;
     if (h->dtype == QG_F32 && h->layers == 1 && h->solver == QG_SOLVER_FFT) {
-        s = refine_psi(h, &scratch, &lo);
+        s = refine_psi(h, &lo);
         if (s != QG_OK) return s;
     }
     s = diagnostics_sums(h, lo, h->stream);
-    if (scratch) cudaFreeAsync(scratch, h->stream);
     if (s != QG_OK) return s;
     QG_TRY(cudaMemcpyAsync(h->hout, h->dout, sizeof(double) * 5, cudaMemcpyDeviceToHost, h->stream));
     QG_TRY(cudaStreamSynchronize(h->stream));

@@ -149,13 +149,17 @@ __global__ void prolong_pair_kernel(const float* c, const float* __restrict__ d,
     const float a = (float)(i & (f - 1)) / (float)f, b = (float)(j & (f - 1)) / (float)f;
     const float wt[4] = {(1.0f - a) * (1.0f - b), a * (1.0f - b), (1.0f - a) * b, a * b};   // exact
     const size_t o = (size_t)J * ldc + I;
-    const long long cn = (long long)((ny >> levels) + 1) * ldc;
+    const int mx = nx >> levels, my = ny >> levels;
+    const long long cn = (long long)(my + 1) * ldc;
     (void)cn;
     float s = 0.0f, e = 0.0f;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const size_t q = o + (k & 1) + (size_t)(k >> 1) * ldc;
-        if (wt[k] == 0.0f || !QG_IN((long long)q, cn, 105)) continue;   // (off the grid at the walls)
+        // (past the grid, or a wall: zero, whatever a solve left there)
+        const int In = I + (k & 1), Jn = J + (k >> 1);
+        if (wt[k] == 0.0f || In == 0 || Jn == 0 || In >= mx || Jn >= my || !QG_IN((long long)q, cn, 105))
+            continue;
         const float x = c[q], p = __fmul_rn(wt[k], x);
         const float t = __fadd_rn(s, p), z = __fsub_rn(t, s);
         e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z)));
