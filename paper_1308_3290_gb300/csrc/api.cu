@@ -2318,9 +2318,11 @@ qg_status qg_tape_begin(qg_handle h, int64_t every, int64_t max_steps) {
     // tape), else an allocation of the tape's own
     const size_t bytes = h->plane_f * h->esz;
     const size_t nck = (size_t)(max_steps / every) + 1, nseg = every > 1 ? (size_t)every + 1 : 0;
-    const size_t total = (nck + nseg + (every > 1 ? 1 : 0)) * bytes + 4 * sizeof(double);
+    // (counts whose bytes do not fit a size_t are more than any memory)
+    const size_t most = SIZE_MAX / 4 / bytes;
+    bool ok = nck <= most && nseg <= most;
+    const size_t total = ok ? (nck + nseg + (every > 1 ? 1 : 0)) * bytes + 4 * sizeof(double) : 0;
     tp->pooled = total <= kTapePool;
-    bool ok = true;
     for (int k = 0; k < AdjWork::NBUF && ok; ++k)
         if (!h->adj.buf[k]) ok = dev_alloc(h, &h->adj.buf[k], bytes) == QG_OK;
     if (ok && h->levels && !h->adj.part)
