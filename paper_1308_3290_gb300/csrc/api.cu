@@ -1272,10 +1272,23 @@ qg_status build_graph(qg_ctx* h) {
     return QG_OK;
 }
 
+// Whether the caller is capturing the handle's stream.
+bool stream_captured(qg_ctx* h) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
 // Run `body` (a qg_status of the stream it enqueues on) on the handle's
-// stream: as it is the first time, from a captured graph after that.
+// stream: as it is the first time, from a captured graph after that.  While
+// the caller captures the stream, as it is: a graph cannot be launched into
+// another's capture.
 template <typename F>
 qg_status replay(qg_ctx* h, Replay& r, F body) {
+    if (stream_captured(h)) return body(h->stream);
     if (!r.exec && ++r.uses > 1) {
         QG_TRY(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
         const qg_status st = body(h->cap);
