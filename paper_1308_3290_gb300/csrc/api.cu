@@ -1627,7 +1627,10 @@ qg_status qg_set_forcing(qg_handle h, const void* forcing) {
 // handle's own: the default pool gives its memory back to the driver at
 // every synchronisation, and taking it again cost 200 us a call.  The pool
 // holds no more than the largest call used and goes with the handle.
+// (While the caller captures the stream the memory belongs to the caller's
+// graph, and a pool cannot be made.)
 static cudaError_t scratch_alloc(qg_ctx* h, void** p, size_t bytes) {
+    if (stream_captured(h)) return cudaMallocAsync(p, bytes, h->stream);
     if (!h->pool) {
         cudaMemPoolProps pp = {};
         pp.allocType = cudaMemAllocationTypePinned;

@@ -1,6 +1,6 @@
-"""Calls that a program may capture into a CUDA graph of its own: the energy sum and
-the reverse steps, on a handle's first use and after the handle has replayed
-its own graphs, several times in one capture.
+"""Calls that a program may capture into a CUDA graph of its own: the energy sum,
+the reverse steps and the stand-alone operators, on a handle's first use and
+after the handle has replayed its own graphs, several times in one capture.
 The captured work gives what the calls give.  Each case in a process of its
 own: a capture that fails leaves the next one's state undefined."""
 import os
@@ -35,6 +35,13 @@ with torch.cuda.stream(s):
         b.step(12)
         out = [new(127, 63), new(127, 63)]
         call = lambda: (qg.qg_energy_gradient(b.h, 1.0, out[0]), qg.qg_adjoint_step(b.h, 1, out[0], out[1]))
+    else:
+        out = [new(63, 31), new(63, 31), new(127, 63), w.clone()]
+        def call():
+            qg.qg_restrict(b.h, w, out[0], 1)
+            qg.qg_poisson_solve(b.h, out[0], out[1], 1)
+            qg.qg_prolong(b.h, out[1], out[2], 1)
+            qg.qg_restrict(b.h, out[3], out[3], 1)      # overlapping: through scratch
     for _ in range(before):
         call()
     s.synchronize()
@@ -67,7 +74,7 @@ print("SAME")
 """
 
 
-@pytest.mark.parametrize("what", ["energy", "adjoint"])
+@pytest.mark.parametrize("what", ["energy", "adjoint", "operators"])
 @pytest.mark.parametrize("before", [0, 1, 4])
 def test_capture(what, before):
     require_gpu()
