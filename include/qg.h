@@ -403,8 +403,10 @@ qg_status qg_inject_fault(qg_handle h, int kind);
 qg_status qg_tape_begin(qg_handle h, int64_t every, int64_t max_steps);
 
 /* qg_tape_end -- stop recording, free the tape, restore the state (see
- * above).  The work fields of the reversal stay with the handle for its next
- * tape, until qg_destroy.  Safe without a tape.                            */
+ * above).  The work fields of the reversal (12 fields and 4 elliptic ones) stay
+ * with the handle for its next tape, until qg_destroy; so does the memory of
+ * a tape of up to 256 MiB, as scratch for the handle's later calls.  Safe
+ * without a tape.                                                          */
 qg_status qg_tape_end(qg_handle h);
 
 /* qg_adjoint_step -- reverse n steps from the cursor t (n <= t): on entry

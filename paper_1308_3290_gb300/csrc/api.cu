@@ -1623,10 +1623,14 @@ qg_status qg_set_forcing(qg_handle h, const void* forcing) {
     return QG_OK;
 }
 
-// Scratch of one stand-alone call, on the handle's stream, from a pool of the
-// handle's own: the default pool gives its memory back to the driver at
-// every synchronisation, and taking it again cost 200 us a call.  The pool
-// holds no more than the largest call used and goes with the handle.
+constexpr size_t kTapePool = (size_t)256 << 20;
+
+// Scratch of one stand-alone call, and a tape's states up to kTapePool bytes,
+// on the handle's stream from a pool of the handle's own: the default pool
+// gives its memory back to the driver at every synchronisation, and taking it
+// again cost 200 us a call.  The pool keeps what was live at once, up to four of
+// the handle's fields (no call takes more) or kTapePool if that is more, and
+// gives the rest back at the next synchronisation; it goes with the handle.
 // (While the caller captures the stream the memory belongs to the caller's
 // graph, and a pool cannot be made.)
 static cudaError_t scratch_alloc(qg_ctx* h, void** p, size_t bytes) {
@@ -1637,7 +1641,7 @@ static cudaError_t scratch_alloc(qg_ctx* h, void** p, size_t bytes) {
         pp.location.type = cudaMemLocationTypeDevice;
         cudaError_t e = cudaGetDevice(&pp.location.id);
         if (e == cudaSuccess) e = cudaMemPoolCreate(&h->pool, &pp);
-        uint64_t keep = UINT64_MAX;
+        uint64_t keep = std::max<uint64_t>(kTapePool, 4 * (uint64_t)h->plane_f * h->layers * h->esz);
         if (e == cudaSuccess)
             e = cudaMemPoolSetAttribute(h->pool, cudaMemPoolAttrReleaseThreshold, &keep);
         if (e != cudaSuccess) return e;
@@ -2300,8 +2304,6 @@ qg_status energy_gradient(qg_ctx* h, double scale, void* g) {
 }
 
 }  // namespace
-
-constexpr size_t kTapePool = (size_t)256 << 20;
 
 static void tape_release(qg_ctx* h) {
     if (!h->tape) return;
