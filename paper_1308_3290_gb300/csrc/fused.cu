@@ -363,7 +363,7 @@ __device__ __forceinline__ void sweep_tile(const CUtensorMap* tm_w, const CUtens
         // Laplacian joins b on w^(s) in FP64.  In FP32 the two stay apart:
         // their rounded sum left the stage's weights up to half an ulp of b
         // short of one, the same in every step (256 x 512, l = 2, 23 steps:
-        // the state 7.5e-7 off, 2.0e-7 with two products, which cost 2 % of a
+        // the state 7.5e-7 off, 1.8e-7 with two products, which cost 2 % of a
         // 2048 x 4096, l = 2 step)
         constexpr bool kApart = sizeof(T) == 4 && !TL;
         const T c_lap0 = T(-2) * (p.c_lapx + p.c_lapy);
@@ -444,14 +444,20 @@ __device__ __forceinline__ void sweep_tile(const CUtensorMap* tm_w, const CUtens
                     Gv = fma(k_0, v00, Gv);
                     Gv = fma(k_ly, WV[sa][i] + WV[sb][i], Gv);
                     Gv = fma(k_lx, WV[sc][i + 1] + WV[sc][i - 1], Gv);
-                    Gv = fma(p.b, q00, Gv);
                 } else {
                     Gv = fma(k_0, q00, Gv);
                     Gv = fma(k_ly, q01 + q0m, Gv);
                     Gv = fma(k_lx, q10 + qm0, Gv);
-                    if constexpr (kApart) Gv = fma(p.b, q00, Gv);
                 }
-                out[q] = fma(p.a, wn[q], Gv);
+                // FP32: w^n first.  b w^(s) first leaves its rounding at b = 2/3,
+                // which for products with 2/3 has a mean of its own: the state
+                // shrank by 4e-9 a step
+                if constexpr (sizeof(T) == 4) {
+                    out[q] = fma(p.b, q00, fma(p.a, wn[q], Gv));
+                } else {
+                    if constexpr (TL) Gv = fma(p.b, q00, Gv);
+                    out[q] = fma(p.a, wn[q], Gv);
+                }
             }
 
             const bool quad_ok = IN || (row_ok && xq >= 1 && xq + 3 <= nx - 1);

@@ -93,7 +93,7 @@ node_stage_kernel(FusedParams<T> p) {
         jac = fma(q[WX - 1], p01 - pm0, jac);
         jac = fma(-q[1 - WX], p10 - p0m, jac);
         const T beta = fma(T(4), h0, hp + hm);
-        // w^(s+1) = a w^n + b w^(s) + b dt G, the centre's weights as in fused.cu
+        // w^(s+1) = a w^n + b w^(s) + b dt G, the centre's weights and the order as in fused.cu
         constexpr bool kApart = sizeof(T) == 4;
         const T bdt = p.b * dt;
         const T k_lx = p.c_lapx * bdt, k_ly = p.c_lapy * bdt;
@@ -103,8 +103,8 @@ node_stage_kernel(FusedParams<T> p) {
         g = fma(k_0, q00, g);
         g = fma(k_ly, q01 + q0m, g);
         g = fma(k_lx, q10 + qm0, g);
-        if constexpr (kApart) g = fma(p.b, q00, g);
         out = fma(p.a, wn, g);
+        if constexpr (kApart) out = fma(p.b, q00, out);
         if (QG_IN(o, fine_n, 86)) p.wout[o] = out;
     }
     if constexpr (LV > 0) {

@@ -37,3 +37,20 @@ def test_no_drift(monkeypatch, nx, ny, levels, Re, tile):
     b.close()
     drift = float((err * ref).sum() / (ref * ref).sum())
     assert abs(drift) <= 1e-7, drift
+
+
+def test_no_drift_of_ensemble_members():
+    require_gpu()
+    m = [dict(nx=64, ny=128, Re=300.0, Ro=0.0016, levels=1, dt=4e-3 / 64),
+         dict(nx=64, ny=128, Re=800.0, Ro=0.0016, levels=1, dt=4e-3 / 64)]
+    e = qg.Ensemble(m, dtype="f32")
+    w0 = inputs.gyre_state(64, 128, seed=4).astype(np.float32).astype(np.float64)
+    for i in range(2):
+        e.member(i).set_state(w0)
+    e.step(23)
+    for i in range(2):
+        ref = O.run(w0, O.Basin(64, 128, Re=m[i]["Re"], Ro=0.0016, levels=1, dt=4e-3 / 64), 23)
+        err = to_np(e.member(i).state()) - ref
+        drift = float((err * ref).sum() / (ref * ref).sum())
+        assert abs(drift) <= 1e-7, (i, drift)
+    e.close()
