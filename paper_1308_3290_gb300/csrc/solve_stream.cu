@@ -321,9 +321,8 @@ __device__ __forceinline__ void row_bwd(Cplx<T> (&v)[16], CT<T>* row, int j,
 // Columns j = t + G r (r < 8) and c G - t (c = 16 - r) of the right-hand side
 // rows ra and rb (existing: va, vb; planes ia, ib): plane 0, plus plane 2 on
 // rows with row % part_py == 0, plus planes 1 and 3 at columns with column %
-// part_px == 0.  Where the period divides G one test of t serves every column;
-// at 128 intervals G is 16 and the period up to 32 (tiles 64 columns wide, l =
-// 1), and the columns of t = 0 are tested one by one.  Eight columns at a time: the loads of all their planes are in flight
+// part_px == 0.  The periods divide G, so one test of t serves every column.
+// Eight columns at a time: the loads of all their planes are in flight
 // together, within the register budget.
 template <typename T, int LG>
 __device__ __forceinline__ void load_rhs(const SolveParams<T>& P, const T* const (&ia)[4],
@@ -332,7 +331,6 @@ __device__ __forceinline__ void load_rhs(const SolveParams<T>& P, const T* const
     using Q = Half<LG>;
     // (a row that does not exist reads row 0, a wall: zeros)
     const int oa = (va ? ra : 0) * P.ld, ob = (vb ? rb : 0) * P.ld;
-    constexpr int kMaxPeriod = 32;
     const bool cx = P.nin > 1 && (t & (P.part_px - 1)) == 0;
     const bool ya = P.nin > 1 && va && (ra & (P.part_py - 1)) == 0;
     const bool yb = P.nin > 1 && vb && (rb & (P.part_py - 1)) == 0;
@@ -341,10 +339,6 @@ __device__ __forceinline__ void load_rhs(const SolveParams<T>& P, const T* const
         auto col = [&](int r) { return h == 0 ? t + Q::G * r : (8 - r) * Q::G - t; };
         // not a wall (z_0, z_N)
         auto ok = [&](int r) { return (t > 0 || r != 0) && QG_IN(col(r), P.mx, 63); };
-        // a seam's column, given cx
-        auto seam = [&](int r) {
-            return ok(r) && (Q::G >= kMaxPeriod || (col(r) & (P.part_px - 1)) == 0);
-        };
         T a[8], b[8];
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
@@ -355,8 +349,8 @@ __device__ __forceinline__ void load_rhs(const SolveParams<T>& P, const T* const
             T c[8], d[8];
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
-                c[r] = seam(r) ? __ldg(ia[1] + oa + col(r)) : T(0);
-                d[r] = seam(r) ? __ldg(ib[1] + ob + col(r)) : T(0);
+                c[r] = ok(r) ? __ldg(ia[1] + oa + col(r)) : T(0);
+                d[r] = ok(r) ? __ldg(ib[1] + ob + col(r)) : T(0);
             }
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
@@ -369,7 +363,7 @@ __device__ __forceinline__ void load_rhs(const SolveParams<T>& P, const T* const
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
                 c[r] = ok(r) ? __ldg(in[2] + o + col(r)) : T(0);
-                d[r] = cx && seam(r) ? __ldg(in[3] + o + col(r)) : T(0);
+                d[r] = cx && ok(r) ? __ldg(in[3] + o + col(r)) : T(0);
             }
 #pragma unroll
             for (int r = 0; r < 8; ++r) x[r] += c[r] + d[r];
