@@ -321,8 +321,10 @@ __device__ __forceinline__ void row_bwd(Cplx<T> (&v)[16], CT<T>* row, int j,
 // Columns j = t + G r (r < 8) and c G - t (c = 16 - r) of the right-hand side
 // rows ra and rb (existing: va, vb; planes ia, ib): plane 0, plus plane 2 on
 // rows with row % part_py == 0, plus planes 1 and 3 at columns with column %
-// part_px == 0.  The periods divide G, so one test of t serves every column.
-// Eight columns at a time: the loads of all their planes are in flight
+// part_px == 0.  One test of t serves every column where the period divides G.
+// At 128 intervals G is 16 and the period of a 64-column tile at l = 1 is 32:
+// there t = 0 also reads planes 1 and 3 at columns between the seams, where they
+// hold zeros (testing each column cost 4 % of a 256 x 512, l = 1 step).  Eight columns at a time: the loads of all their planes are in flight
 // together, within the register budget.
 template <typename T, int LG>
 __device__ __forceinline__ void load_rhs(const SolveParams<T>& P, const T* const (&ia)[4],

@@ -91,7 +91,9 @@ __global__ void restrict_kernel(const T* __restrict__ fine, int ldf,
         coarse[(size_t)J * ldc + I] = restricted_at(fine, ldf, I, J, my, levels);
 }
 
-// R^l w into a step's partial planes: plane 0 whole, planes 1 to 3 zero.
+// R^l w into a step's partial planes: plane 0 whole, planes 1 to 3 zero at every
+// interior node (the steps write them on their tile's seams only, and the
+// solves count on zeros elsewhere).
 // Launch-bound: member blockIdx.y of an ensemble takes its arrays from the
 // table, so that one launch serves all members (a memset and a restriction
 // each took 460 us for 48 basins, the batched launch some 40 with its wait).
