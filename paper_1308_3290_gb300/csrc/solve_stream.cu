@@ -523,13 +523,19 @@ __device__ __forceinline__ void stream_item(const SolveParams<T>& P, int npairs,
             } else {
                 const T q1 = P.scale * Fa, q2 = P.scale * Fb;
                 const T al = ro * (lxa + ly);
-                // (the determinant al (al - f1 - f2) factor by factor, both
-                // negative: no underflow, and no division, whose rare path
-                // splits the chains of the 16 modes: FP32 256 x 256, l = 0,
-                // 51.4 us a step with two divisions a mode, 43.1 with one)
+                // the two quotients without a division, whose rare path splits
+                // the chains of the 16 modes (FP32 256 x 256, l = 0: 51.4 us a
+                // step with two divisions a mode, 43.1 with one, 36.9 without):
+                // a reciprocal factor by factor, both negative, and the residual
+                // correction of Markstein (1990), which rounds them as a
+                // division would
+                const T den = al * (al - P.f1 - P.f2);
                 const T r = recip(al) * recip(al - P.f1 - P.f2);
-                x = (al * q1 - P.f2 * q1 - P.f1 * q2) * r;
-                y = (al * q2 - P.f2 * q1 - P.f1 * q2) * r;
+                const T n1 = al * q1 - P.f2 * q1 - P.f1 * q2, n2 = al * q2 - P.f2 * q1 - P.f1 * q2;
+                x = n1 * r;
+                y = n2 * r;
+                x = fma(fma(-den, x, n1), r, x);
+                y = fma(fma(-den, y, n2), r, y);
             }
             v[i] = Cplx<T>{x, y};
             // the walls l = 0 and my stay 0
@@ -831,7 +837,7 @@ cudaError_t launch_ppc(const SolveParams<T>& P, int npairs, cudaStream_t s) {
 // with (4, 2, 1).
 // Two layers in FP32 store one value of each layer per pair and element, 8
 // bytes: the two passes that write the scratch arrays take four pairs at
-// least, a 32-byte sector (l = 0, 1024 x 2048: 182 us with (4, 4, 2), 222 with
+// least, a 32-byte sector (l = 0, 1024 x 2048: 183 us with (4, 4, 2), 222 with
 // (1, 1, 1), 197 with (2, 2, 1); 256 x 256 36.9, 39.0 and 39.0).
 template <typename T>
 __host__ __device__ constexpr int ppc_max(int lg) {
