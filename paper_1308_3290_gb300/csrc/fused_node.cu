@@ -45,7 +45,7 @@ node_stage_kernel(FusedParams<T> p) {
     load_halo<T, LV>(p.w, sw, x0, y0, nx, ny, ld);
     T wn = T(0), f = T(0);
     const size_t o = (size_t)y * ld + x;
-    if (in && QG_IN(o, fine_n, 82)) {
+    if (in && QG_IN(o, fine_n, 132)) {
         if (p.a != T(0)) wn = p.wn[o];
         f = p.f2d ? p.f2d[o] : p.frow[y];
     }
@@ -105,7 +105,7 @@ node_stage_kernel(FusedParams<T> p) {
         g = fma(k_lx, q10 + qm0, g);
         out = fma(p.a, wn, g);
         if constexpr (kApart) out = fma(p.b, q00, out);
-        if (QG_IN(o, fine_n, 86)) p.wout[o] = out;
+        if (QG_IN(o, fine_n, 136)) p.wout[o] = out;
     }
     if constexpr (LV > 0) {
         so[threadIdx.x] = out;

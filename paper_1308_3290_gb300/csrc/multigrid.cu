@@ -357,6 +357,9 @@ __global__ void __launch_bounds__(256) mg_sum_kernel(MGSumParams<T> q) {
         const int i = e & (q.mx - 1), j = e >> lx;
         if (i < 1 || j < 1) continue;
         const size_t o = (size_t)j * q.ld_in + i;
+        if (!(QG_IN((long long)o, (long long)(q.my + 1) * q.ld_in, 90) &&
+              QG_IN((long long)j * q.ld + i, (long long)(q.my + 1) * q.ld, 90)))
+            continue;
         T v = q.in[0][o];
         for (int k = 1; k < q.nin; ++k) v = v + q.in[k][o];
         q.rhs[(size_t)j * q.ld + i] = v;

@@ -32,7 +32,7 @@ __device__ __forceinline__ void load_halo(const T* src, T* dst, int x0, int y0, 
     for (int e = threadIdx.x; e < Q::WY * Q::WX; e += Q::THREADS) {
         const int hx = x0 - 1 + e % Q::WX, hy = y0 - 1 + e / Q::WX;
         const bool ok = hx >= 0 && hx <= nx && hy >= 0 && hy <= ny &&
-                        QG_IN((long long)hy * ld + hx, (long long)(ny + 1) * ld, 81);
+                        QG_IN((long long)hy * ld + hx, (long long)(ny + 1) * ld, 131);
         dst[e] = ok ? src[(size_t)hy * ld + hx] : T(0);
     }
 }
@@ -46,7 +46,7 @@ __device__ __forceinline__ void load_patch(const T* src, T* cp, int x0, int y0, 
     for (int e = threadIdx.x; e < Q::CX * Q::CY; e += Q::THREADS) {
         const int I = I0 + e % Q::CX, J = J0 + e / Q::CX;
         const bool ok = I >= 0 && I <= mx && J >= 0 && J <= my &&
-                        QG_IN((long long)J * ldp + I, (long long)(my + 1) * ldp, 83);
+                        QG_IN((long long)J * ldp + I, (long long)(my + 1) * ldp, 133);
         cp[e] = ok ? src[(size_t)J * ldp + I] : T(0);
     }
 }
@@ -63,7 +63,7 @@ __device__ __forceinline__ void prolong_halo(const T* cp, T* cr, T* sp) {
     for (int e = threadIdx.x; e < Q::WY * Q::CX; e += Q::THREADS) {
         const int r = e / Q::CX, c = e % Q::CX;
         const int b = (F - 1 + r) / F, ph = (F - 1 + r) % F;
-        const bool ok = QG_IN((b + 1) * Q::CX + c, Q::CX * Q::CY, 84);
+        const bool ok = QG_IN((b + 1) * Q::CX + c, Q::CX * Q::CY, 134);
         const T lo = ok ? cp[b * Q::CX + c] : T(0), hi = ok ? cp[(b + 1) * Q::CX + c] : T(0);
         const T wt = T(ph) * (T(1) / T(F));
         cr[e] = ph == 0 ? lo : fma(wt, hi, (T(1) - wt) * lo);
@@ -72,7 +72,7 @@ __device__ __forceinline__ void prolong_halo(const T* cp, T* cr, T* sp) {
     for (int e = threadIdx.x; e < Q::WY * Q::WX; e += Q::THREADS) {
         const int r = e / Q::WX, c = e % Q::WX;
         const int a = (F - 1 + c) / F, ph = (F - 1 + c) % F;
-        const bool ok = QG_IN(r * Q::CX + a + 1, Q::WY * Q::CX, 85);
+        const bool ok = QG_IN(r * Q::CX + a + 1, Q::WY * Q::CX, 135);
         const T lo = ok ? cr[r * Q::CX + a] : T(0), hi = ok ? cr[r * Q::CX + a + 1] : T(0);
         const T wt = T(ph) * (T(1) / T(F));
         sp[e] = ph == 0 ? lo : fma(wt, hi, (T(1) - wt) * lo);
@@ -87,7 +87,7 @@ __device__ __forceinline__ T prolong_own(const T* cp, int i, int j) {
     constexpr int F = Q::F;
     const T* c = cp + (1 + j / F) * Q::CX + 1 + i / F;
     const T a = T(i % F) * (T(1) / T(F)), b = T(j % F) * (T(1) / T(F));
-    if (!QG_IN((2 + j / F) * Q::CX + 2 + i / F, Q::CX * Q::CY, 84)) return T(0);
+    if (!QG_IN((2 + j / F) * Q::CX + 2 + i / F, Q::CX * Q::CY, 134)) return T(0);
     const T lo = fma(a, c[1], (T(1) - a) * c[0]);
     const T hi = fma(a, c[Q::CX + 1], (T(1) - a) * c[Q::CX]);
     return fma(b, hi, (T(1) - b) * lo);
@@ -110,7 +110,7 @@ __device__ __forceinline__ void restrict_tile(const T* so, T* sx, T* const (&par
 #pragma unroll
         for (int d = -(F - 1); d < F; ++d) {
             const int k = c * F + d;
-            if (k >= 0 && k < NX && QG_IN(r * NX + k, NY * NX, 87))
+            if (k >= 0 && k < NX && QG_IN(r * NX + k, NY * NX, 137))
                 v = fma(T(F - (d < 0 ? -d : d)) * (T(1) / T(F * F)), so[r * NX + k], v);
         }
         sx[e] = v;
@@ -122,13 +122,13 @@ __device__ __forceinline__ void restrict_tile(const T* so, T* sx, T* const (&par
 #pragma unroll
         for (int d = -(F - 1); d < F; ++d) {
             const int r = m * F + d;
-            if (r >= 0 && r < NY && QG_IN(r * Q::SX + c, NY * Q::SX, 88))
+            if (r >= 0 && r < NY && QG_IN(r * Q::SX + c, NY * Q::SX, 138))
                 v = fma(T(F - (d < 0 ? -d : d)) * (T(1) / T(F * F)), sx[r * Q::SX + c], v);
         }
         const int I = (x0 >> LV) + c, J = (y0 >> LV) + m;
         const int pl = (c == Q::SX - 1 ? 1 : 0) + (m == Q::SY - 1 ? 2 : 0);
         if (I >= 1 && I <= mx - 1 && J >= 1 && J <= my - 1 &&
-            QG_IN((long long)J * ldc + I, (long long)(my + 1) * ldc, 89))
+            QG_IN((long long)J * ldc + I, (long long)(my + 1) * ldc, 139))
             part[pl][(size_t)J * ldc + I] = v;
     }
 }

@@ -55,7 +55,7 @@ __device__ __forceinline__ T sine_sum(const T* S, const T* u, const T* v, int N,
     for (int n = 0; n < h; n += 4) {
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            if (QG_IN((n + q) * N + k, h * N, 91)) a[q] = fma(S[(n + q) * N + k], x[n + q + 1], a[q]);
+            if (QG_IN((n + q) * N + k, h * N, 121)) a[q] = fma(S[(n + q) * N + k], x[n + q + 1], a[q]);
     }
     return (a[0] + a[2]) + (a[1] + a[3]);
 }
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(kMaxN) dense_x_kernel(SolveParams<T> P, const 
     pdl_trigger();
     const long long n = (long long)(P.my + 1) * P.ld;
     (void)n;
-    if (k >= 1 && k < N && QG_IN((long long)r * P.ld + k, n, 92)) {
+    if (k >= 1 && k < N && QG_IN((long long)r * P.ld + k, n, 122)) {
         const size_t o = (size_t)r * P.ld + k;
         T x;
         if (FWD) {
@@ -120,9 +120,9 @@ __global__ void __launch_bounds__(kMaxN) dense_x_kernel(SolveParams<T> P, const 
         const long long nt = (long long)(P.mx + 1) * P.ld_tr;
         (void)nt;
         if (FWD) {
-            if (QG_IN((long long)k * P.ld_tr + r, nt, 93))
+            if (QG_IN((long long)k * P.ld_tr + r, nt, 123))
                 (L ? P.tr[1] : P.tr[0])[(size_t)k * P.ld_tr + r] = F;
-        } else if (QG_IN((long long)r * P.ld + k, n, 94)) {
+        } else if (QG_IN((long long)r * P.ld + k, n, 124)) {
             (L ? P.out[1] : P.out[0])[(size_t)r * P.ld + k] = F;
         }
     }
@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(kMaxN) dense_y_kernel(SolveParams<T> P, const 
     pdl_trigger();
     const long long nt = (long long)(P.mx + 1) * P.ld_tr;
     (void)nt;
-    if (in && QG_IN((long long)k * P.ld_tr + l, nt, 95)) {
+    if (in && QG_IN((long long)k * P.ld_tr + l, nt, 125)) {
 #pragma unroll
         for (int L = 0; L < NL; ++L) f[L][l] = P.tr[L][(size_t)k * P.ld_tr + l];
     }
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kMaxN) dense_y_kernel(SolveParams<T> P, const 
     __syncthreads();
     const long long n = (long long)(P.my + 1) * P.ld;
     (void)n;
-    if (in && QG_IN((long long)l * P.ld + k, n, 96)) {
+    if (in && QG_IN((long long)l * P.ld + k, n, 126)) {
 #pragma unroll
         for (int L = 0; L < NL; ++L)
             P.work[L][(size_t)l * P.ld + k] = sine_sum(tab, u[L], v[L], N, l);

@@ -108,7 +108,8 @@ __global__ void __launch_bounds__(256) init_partials_kernel(InitPartials<T> one,
         const size_t o = (size_t)J * q.ldc + I;
         if (!QG_IN((long long)o, (long long)(q.my + 1) * q.ldc, 42)) continue;
         q.part[o] = restricted_at(q.w, q.ldf, I, J, q.my, q.levels);
-        for (int k = 1; k < 4; ++k) q.part[k * q.plane + o] = T(0);
+        for (int k = 1; k < 4; ++k)
+            if (QG_IN((long long)o, (long long)q.plane, 46)) q.part[k * q.plane + o] = T(0);
     }
 }
 
@@ -131,12 +132,15 @@ __global__ void prolong_kernel(const T* __restrict__ coarse, int ldc,
     // the coarse grid has my + 1 rows of pitch ldc
     if (!DENSE && !QG_IN((long long)(J + 1) * ldc + I + 1, (long long)(my + 1) * ldc, 43)) return;
     auto at = [&](int di, int dj) {
-        if (DENSE && !(I + di >= 1 && I + di < mx && J + dj >= 1 && J + dj < my)) return T(0);
+        if (DENSE && !(I + di >= 1 && I + di < mx && J + dj >= 1 && J + dj < my &&
+                       QG_IN((long long)(J + dj - 1) * ldc + I + di - 1, (long long)(my - 1) * ldc, 43)))
+            return T(0);
         return C[(size_t)dj * ldc + di];
     };
     const T v = (T(1) - a) * (T(1) - b) * at(0, 0) + a * (T(1) - b) * at(1, 0) +
                 (T(1) - a) * b * at(0, 1) + a * b * at(1, 1);
-    if (DENSE || QG_IN((long long)j * ldf + i, (long long)(ny + 1) * ldf, 44))
+    if (DENSE ? QG_IN((long long)(j - 1) * ldf + i - 1, (long long)(ny - 1) * ldf, 44)
+              : QG_IN((long long)j * ldf + i, (long long)(ny + 1) * ldf, 44))
         fine[(size_t)j * ldf + i] = v;
 }
 
@@ -246,6 +250,9 @@ __device__ __forceinline__ void cfl_max(const T* __restrict__ psi, int ldp, int 
         if constexpr (LV == 0) {   // the fine psi itself: one node per thread
             if (I < 1 || J < 1) continue;
             const T* p = psi + (size_t)J * ldp + I;
+            if (!(QG_IN((long long)(J - 1) * ldp + I, (long long)(ny + 1) * ldp, 47) &&
+                  QG_IN((long long)(J + 1) * ldp + I, (long long)(ny + 1) * ldp, 47)))
+                continue;
             ax = fmax(ax, fabs(p[1] - p[-1]));
             ay = fmax(ay, fabs(p[ldp] - p[-ldp]));
             continue;
@@ -256,7 +263,8 @@ __device__ __forceinline__ void cfl_max(const T* __restrict__ psi, int ldp, int 
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int Jr = J - 1 + r, Iq = I - 1 + q;
-                c[r][q] = (Jr >= 0 && Jr <= my && Iq >= 0 && Iq <= mx)
+                c[r][q] = (Jr >= 0 && Jr <= my && Iq >= 0 && Iq <= mx &&
+                           QG_IN((long long)Jr * ldp + Iq, (long long)(my + 1) * ldp, 47))
                               ? psi[(size_t)Jr * ldp + Iq] : T(0);
             }
         T row[3][W];
@@ -320,6 +328,7 @@ template <typename T>
 __device__ __forceinline__ void accumulate(double* __restrict__ acc, const T* __restrict__ src,
                                            int n) {
     for (int e = 4 * (blockIdx.x * blockDim.x + threadIdx.x); e < n; e += 4 * gridDim.x * blockDim.x) {
+        if (!QG_IN(e + 3, n, 45)) break;   // (n is a multiple of 4)
         T v[4];
         if constexpr (sizeof(T) == 4) {
             const float4 q = *reinterpret_cast<const float4*>(src + e);
