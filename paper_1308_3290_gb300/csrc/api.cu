@@ -2412,8 +2412,8 @@ qg_status qg_energy_gradient(qg_handle h, double scale, void* g) {
 //   * one fused fine-stage launch per CGP level among the group's members,
 //     over all their tiles, each CTA reading its member's tensor maps and
 //     parameters from a device table.
-// Within a branch the launches follow each other with programmatic
-// dependent launch, as in a single basin's step.
+// Within a branch the launches follow each other without programmatic
+// dependent launch (kEnsemblePdl).
 
 #define QG_TRY_E(expr)                        \
     do {                                      \

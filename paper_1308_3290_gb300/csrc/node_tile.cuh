@@ -1,6 +1,6 @@
 // Tiles of 16 x 8 fine nodes (16 x 16 at l = 4), one thread per node: the
 // staging, prolongation and restriction that the kernels of fused_node.cu and
-// adjoint_node.cu share.
+// adjoint.cu share.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -32,7 +32,7 @@ struct DstLaunch {
     int lanes;
 };
 
-// ---- kernels (declared here, defined in dst.cu / stencil.cu / diag.cu) ----
+// ---- kernels (declared here, defined in solve*.cu / stencil.cu / diag.cu) ----
 
 // The elliptic solve of one level (solve.cu): x pass of `in` (the sum of
 // nin planes per layer; with nin == 4 plane 1 counts at columns k % part_px
@@ -188,7 +188,7 @@ struct AdjParams {
     int nx, ny, ld;
     T c_jac, c_beta;      // 1/(12 dx dy), 1/(12 Ro dx)
     T c_lapx, c_lapy;     // 1/(Re dx^2), 1/(Re dy^2)
-    T dt, a, b;           // time step and the stage's TVDRK3 weights
+    T dt, b;              // time step and the stage's TVDRK3 weight
     T inv_dx2, inv_dy2, dxdy;
 };
 // Where a source goes: restricted into partial planes of pitch ldc (levels

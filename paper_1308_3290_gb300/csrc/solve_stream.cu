@@ -706,7 +706,7 @@ stream_kernel(SolveParams<T> Pin, int npairs, int cpm) {
 
 // Pairs per y item of the work queue (twice as many per x item, half as
 // long) and its CTA size.
-__host__ __device__ constexpr int queue_ppc(int lgx) { return lgx <= 9 ? 4 : lgx == 10 ? 4 : 2; }
+__host__ __device__ constexpr int queue_ppc(int lgx) { return lgx <= 10 ? 4 : 2; }
 __host__ __device__ constexpr int queue_threads(int lgx) {
     return round32(9 * (1 << (lgx + 1)) / 256 * queue_ppc(lgx));
 }
