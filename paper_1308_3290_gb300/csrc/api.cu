@@ -394,8 +394,7 @@ qg_status get_level(qg_ctx* h, int lv, const LevelTables** out) {
     for (int l = 1; l < t.my; ++l) ly[l] = (2.0 * std::cos(pi * l / t.my) - 2.0) / (t.dyc * t.dyc);
     s = upload_real(h, &t.lamx, lx);
     if (s == QG_OK) s = upload_real(h, &t.lamy, ly);
-    // the tables of engines 50 and 42, one upload each (their parts start on
-    // 16 bytes: even counts)
+    // engine 50's tables, one upload (its parts start on 16 bytes: even counts)
     if (s == QG_OK && stream_supports(t.mx, t.my, h->esz)) {
         const size_t nx = half_table_size(2 * t.mx), ny = half_table_size(2 * t.my);
         const size_t nl = (size_t)9 * (t.my / 8), nm = nx > ny ? nx : ny;
@@ -414,14 +413,6 @@ qg_status get_level(qg_ctx* h, int lv, const LevelTables** out) {
         s = upload_real(h, &t.htx, v);
         t.hty = static_cast<char*>(t.htx) + 2 * nx * h->esz;
         t.lamyr = static_cast<char*>(t.htx) + 2 * (nx + ny) * h->esz;
-    }
-    if (s == QG_OK && !h->member && dense_supports(t.mx, t.my)) {
-        const size_t nx = (size_t)t.mx * t.mx / 2, ny = (size_t)t.my * t.my / 2;
-        std::vector<double> v(nx + ny);
-        dense_table(t.mx, v.data());
-        dense_table(t.my, v.data() + nx);
-        s = upload_real(h, &t.dsx, v);
-        t.dsy = static_cast<char*>(t.dsx) + nx * h->esz;
     }
     if (s != QG_OK) return s;
     h->tables[lv] = t;
@@ -638,6 +629,22 @@ qg_status solve_level(qg_ctx* h, const LevelTables& t, const void* in, void* tr,
     }
     QG_TRY(launch_solve<T>(P, eng, s));
     return QG_OK;
+}
+
+// Engine 42's sine tables of the step's level, one upload: made when the engine
+// is timed or chosen (up to 0.1 ms of a handle's creation).  Not for ensemble
+// members, whose batches it does not solve.
+qg_status dense_tables(qg_ctx* h) {
+    LevelTables& t = h->tables[h->levels];
+    if (t.dsx || h->member || !dense_supports(t.mx, t.my)) return QG_OK;
+    const size_t nx = (size_t)t.mx * t.mx / 2, ny = (size_t)t.my * t.my / 2;
+    std::vector<double> v(nx + ny);
+    dense_table(t.mx, v.data());
+    dense_table(t.my, v.data() + nx);
+    const qg_status s = upload_real(h, &t.dsx, v);
+    if (s == QG_OK) t.dsy = static_cast<char*>(t.dsx) + nx * h->esz;
+    else t.dsx = nullptr;
+    return s;
 }
 
 // ---- solve-engine autotuner ---------------------------------------------
@@ -906,6 +913,7 @@ qg_status autotune_solve(qg_ctx* h) {
     const char* force = std::getenv("QG_SOLVE_ENGINE");
     if (force) {
         const int e = std::atoi(force);
+        if (e == kDenseEngine) QG_TRY_S(dense_tables(h));
         if (engine_ok(h, t, sizeof(T), e)) {
             h->solve_engine = e;
             h->engine_forced = true;
@@ -919,6 +927,7 @@ qg_status autotune_solve(qg_ctx* h) {
         auto it = g_tune_cache.find(key);
         const Tile cached{it == g_tune_cache.end() ? 0 : it->second.rows,
                           it == g_tune_cache.end() ? 0 : it->second.ry};
+        if (it != g_tune_cache.end() && it->second.engine == kDenseEngine) QG_TRY_S(dense_tables(h));
         if (it != g_tune_cache.end() && engine_ok(h, t, sizeof(T), it->second.engine) &&
             !(force && it->second.engine == kDenseEngine) &&
             std::find(tiles.begin(), tiles.end(), cached) != tiles.end()) {
@@ -927,6 +936,7 @@ qg_status autotune_solve(qg_ctx* h) {
             return QG_OK;
         }
     }
+    if (!force) QG_TRY_S(dense_tables(h));
     const std::vector<int> engines = timed_engines(h, t, sizeof(T), !force);
     const int best = fastest((int)engines.size(),
                              [&](int k, int n) { return time_steps<T>(h, engines[k], n); });
