@@ -2351,10 +2351,15 @@ qg_status qg_tape_begin(qg_handle h, int64_t every, int64_t max_steps) {
     bool ok = nck <= most && nseg <= most;
     const size_t total = ok ? (nck + nseg + (every > 1 ? 1 : 0)) * bytes + 4 * sizeof(double) : 0;
     tp->pooled = total <= kTapePool;
-    for (int k = 0; k < AdjWork::NBUF && ok; ++k)
-        if (!h->adj.buf[k]) ok = dev_alloc(h, &h->adj.buf[k], bytes) == QG_OK;
-    if (ok && h->levels && !h->adj.part)
-        ok = dev_alloc(h, &h->adj.part, 4 * h->plane_c * h->esz) == QG_OK;
+    if (ok && !h->adj.buf[0]) {
+        // (one allocation: thirteen took 0.25 ms to free; a field is a multiple
+        // of 128 bytes)
+        void* block = nullptr;
+        ok = dev_alloc(h, &block, AdjWork::NBUF * bytes + (h->levels ? 4 * h->plane_c * h->esz : 0)) == QG_OK;
+        for (int k = 0; k < AdjWork::NBUF && ok; ++k)
+            h->adj.buf[k] = static_cast<char*>(block) + k * bytes;
+        if (ok && h->levels) h->adj.part = static_cast<char*>(block) + AdjWork::NBUF * bytes;
+    }
     if (ok)
         ok = (tp->pooled ? scratch_alloc(h, &tp->block, total) : cudaMalloc(&tp->block, total)) ==
              cudaSuccess;
