@@ -2350,7 +2350,8 @@ qg_status qg_tape_begin(qg_handle h, int64_t every, int64_t max_steps) {
     const size_t most = SIZE_MAX / 4 / bytes;
     bool ok = nck <= most && nseg <= most;
     const size_t total = ok ? (nck + nseg + (every > 1 ? 1 : 0)) * bytes + 4 * sizeof(double) : 0;
-    tp->pooled = total <= kTapePool;
+    // (a tape outlives a caller's capture, and is refused in one)
+    tp->pooled = total <= kTapePool && !stream_captured(h);
     if (ok && !h->adj.buf[0]) {
         // (one allocation: thirteen took 0.25 ms to free; a field is a multiple
         // of 128 bytes)

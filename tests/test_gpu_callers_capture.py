@@ -81,3 +81,35 @@ def test_capture(what, before):
     r = subprocess.run([sys.executable, "-c", _SCRIPT, what, str(before)], cwd=ROOT, capture_output=True,
                        text=True, timeout=300)
     assert r.returncode == 0 and "SAME" in r.stdout, r.stdout[-500:] + r.stderr[-2500:]
+
+
+def test_a_tape_is_not_begun_in_a_capture():
+    """Its states have to outlive the caller's graph: refused, for a handle that
+    has reversed a tape before too, and the handle goes on."""
+    require_gpu()
+    script = """
+import torch
+from paper_1308_3290_gb300 import inputs, qg
+s = torch.cuda.Stream()
+with torch.cuda.stream(s):
+    b = qg.Basin(64, 128, Re=200.0, Ro=0.0016, levels=1, dt=1e-4, dtype="f32")
+    b.set_state(inputs.gyre_state(64, 128, seed=1))
+    qg.qg_tape_begin(b.h, 1, 4)
+    qg.qg_tape_end(b.h)
+    b.synchronize()
+    g = torch.cuda.CUDAGraph()
+    status = None
+    try:
+        with torch.cuda.graph(g, stream=s):
+            try:
+                qg.qg_tape_begin(b.h, 1, 4)
+            except qg.QGError as e:
+                status = e.status
+                raise
+    except Exception:
+        pass
+    assert status == qg.QG_ERR_OOM, status
+print("REFUSED")
+"""
+    r = subprocess.run([sys.executable, "-c", script], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert "REFUSED" in r.stdout, r.stdout[-500:] + r.stderr[-2500:]
